@@ -193,19 +193,23 @@ int build_chunks(ws_ctx* c, int config) {
 }
 bool mixed(const ws_ctx* c) { return c->opts.precision == WS_PREC_MIXED; }
 
-// one RHS evaluation of the stage state Us into the face arrays
-int rhs_faces(ws_ctx* c, double* Us) {
+// The start of an RHS evaluation of the stage state Us: ghost layers and the
+// primitive cache.  FP64: one launch, which also takes the CFL rate into lmax
+// (nullable, zeroed before) and sets the counter *clear (nullable) to zero.
+int rhs_faces(ws_ctx* c, double* Us, unsigned long long* lmax = nullptr, unsigned long long* clear = nullptr) {
   const GridDev& g = c->gd;
+  if (!mixed(c)) {
+    KScope k(c, WS_K_PRIM);
+    launch_prep(g, Us, c->Q, lmax, clear, c->stream);
+    return check_launch(c, "ghost/prim");
+  }
   {
     KScope k(c, WS_K_GHOST, g.ndim);
     for (int d = 0; d < g.ndim; ++d) launch_ghost(g, Us, d, c->stream);
   }
   {
     KScope k(c, WS_K_PRIM);
-    if (mixed(c))
-      launch_prim32(g, Us, c->Q32, c->stream);
-    else
-      launch_prim(g, Us, c->Q, c->stream);
+    launch_prim32(g, Us, c->Q32, c->stream);
   }
   return check_launch(c, "ghost/prim");
 }
@@ -213,24 +217,26 @@ int rhs_faces(ws_ctx* c, double* Us) {
 int faces(ws_ctx* c, int stage_slot) {
   const GridDev& g = c->gd;
   uint8_t* mbase = c->mask + (int64_t)stage_slot * c->nmask;
+  if (!mixed(c)) {
+    KScope k(c, WS_K_FACE);
+    uint8_t* const m[3] = {mbase + c->mask_off[0], mbase + c->mask_off[1], mbase + c->mask_off[2]};
+    launch_face_fp64(g, c->Q, c->Fh, c->us, m, c->opts.eps, c->opts.mood, c->opts.weights, c->stream);
+    return check_launch(c, "face sweep");
+  }
   for (int d = 0; d < g.ndim; ++d) {
     KScope k(c, WS_K_FACE);
-    if (mixed(c))
-      launch_face_mixed(g, d, c->Q32, c->Fh32[d], c->us32[d], mbase + c->mask_off[d], (float)c->opts.eps,
-                        c->opts.mood, c->opts.weights, c->stream);
-    else
-      launch_face_fp64(g, d, c->Q, c->Fh[d], c->us[d], mbase + c->mask_off[d], c->opts.eps, c->opts.mood,
-                       c->opts.weights, c->stream);
+    launch_face_mixed(g, d, c->Q32, c->Fh32[d], c->us32[d], mbase + c->mask_off[d], (float)c->opts.eps, c->opts.mood,
+                      c->opts.weights, c->stream);
   }
   return check_launch(c, "face sweep");
 }
 
-int update(ws_ctx* c, int stage, const double* Un, const double* Us, double* Uout) {
+int update(ws_ctx* c, int stage, const double* Un, const double* Us, double* Uout, double dt = 0.0) {
   KScope k(c, WS_K_UPDATE);
   if (mixed(c))
     launch_update_mixed(c->gd, stage, Un, Us, Uout, c->Fh32, c->us32, c->Q32, c->dt_dev, c->nbad, c->stream);
   else
-    launch_update(c->gd, stage, Un, Us, Uout, c->Fh, c->us, c->dt_dev, c->nbad, c->stream);
+    launch_update(c->gd, stage, Un, Us, Uout, c->Fh, c->us, dt, c->opts.cfl, c->lmax, c->dt_dev, c->nbad, c->stream);
   return check_launch(c, "update");
 }
 
@@ -337,8 +343,8 @@ int step_device(ws_ctx* c, double* U, double dt) {
   const GridDev& g = c->gd;
   int rc;
   c->nbad_last = c->nbad;
-  // a plain fused step clears (or rotates) its own counter
-  if (!(c->fused && !c->learned_on)) CK(c, cudaMemsetAsync(c->nbad, 0, sizeof(unsigned long long), c->stream));
+  // a plain fused step clears (or rotates) its own counter, an FP64 grid step its own
+  if (!(c->fused && !c->learned_on) && (mixed(c) || tubes(c))) CK(c, cudaMemsetAsync(c->nbad, 0, sizeof(unsigned long long), c->stream));
   if (tubes(c) && mixed(c)) {
     const int64_t nt = c->td.ntubes;
     CK(c, cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long) * nt, c->stream));
@@ -393,6 +399,21 @@ int step_device(ws_ctx* c, double* U, double dt) {
     c->last_stages = 3;
     return WS_OK;
   }
+  if (!mixed(c)) {
+    // three launches per stage.  Stage 0's first zeroes the inadmissible-cell
+    // count and takes the CFL rate, its update derives dt; stage 1's first
+    // zeroes the rate for the next step.
+    for (int s = 0; s < 3; ++s) {
+      double* Us = s == 0 ? U : c->S1;
+      if ((rc = rhs_faces(c, Us, s == 0 && dt <= 0.0 ? c->lmax : nullptr,
+                          s == 0 ? c->nbad : (s == 1 ? c->lmax : nullptr))))
+        return rc;
+      if ((rc = faces(c, s))) return rc;
+      if ((rc = update(c, s, U, Us, s == 2 ? U : c->S1, dt))) return rc;
+    }
+    c->last_stages = 3;
+    return WS_OK;
+  }
   for (int s = 0; s < 3; ++s) {
     double* Us = s == 0 ? U : c->S1;
     if ((rc = rhs_faces(c, Us))) return rc;
@@ -400,10 +421,7 @@ int step_device(ws_ctx* c, double* U, double dt) {
       if (dt <= 0.0) {
         CK(c, cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long), c->stream));
         KScope k(c, WS_K_CFL);
-        if (mixed(c))
-          launch_cfl32(g, c->Q32, c->lmax, c->stream);
-        else
-          launch_cfl(g, c->Q, c->lmax, c->stream);
+        launch_cfl32(g, c->Q32, c->lmax, c->stream);
       }
       KScope k(c, WS_K_CFL);
       launch_set_dt(nullptr, dt, c->opts.cfl, c->lmax, c->dt_dev, 1, c->stream);
@@ -607,6 +625,10 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
     rc = fail(c, WS_ECUDA, "copying mask offsets failed");
     goto bad;
   }
+  if (cudaMemset(c->lmax, 0, sizeof(unsigned long long)) != cudaSuccess) {  // FP64 grid steps leave it at zero
+    rc = fail(c, WS_ECUDA, "cudaMemset failed");
+    goto bad;
+  }
   // tube masks hold one byte per padded cell; the bytes that carry no face stay 0xff
   if (cudaMemset(c->mask, tb ? 0xff : 0, 3 * c->nmask) != cudaSuccess) {
     rc = fail(c, WS_ECUDA, "cudaMemset failed");
@@ -662,19 +684,17 @@ int ws_cfl_dt(ws_ctx* c, double* U, double* dt) {
     CK(c, cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long) * n, c->stream));
     launch_tubes_cfl(c->td, c->Q, c->lmax, c->stream);
   } else {
-    int rc = rhs_faces(c, U);
-    if (rc) return rc;
     CK(c, cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long), c->stream));
-    if (mixed(c))
-      launch_cfl32(c->gd, c->Q32, c->lmax, c->stream);
-    else
-      launch_cfl(c->gd, c->Q, c->lmax, c->stream);
+    int rc = rhs_faces(c, U, c->lmax);
+    if (rc) return rc;
+    if (mixed(c)) launch_cfl32(c->gd, c->Q32, c->lmax, c->stream);
   }
   launch_set_dt(nullptr, 0.0, c->opts.cfl, c->lmax, c->dt_dev, n, c->stream);
   int rc = check_launch(c, "cfl");
   if (rc) return rc;
   std::vector<double> h(n);
   CK(c, cudaMemcpyAsync(h.data(), c->dt_dev, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
+  CK(c, cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long) * n, c->stream));  // an FP64 grid step starts from zero
   CK(c, cudaStreamSynchronize(c->stream));
   double m = h[0];
   for (int64_t i = 1; i < n; ++i) m = h[i] < m ? h[i] : m;

@@ -5,11 +5,15 @@
 // evaluation of the same formulas bit for bit.
 #include <cuda_runtime.h>
 
+#include "fp64_pipes.cuh"
 #include "ws_internal.h"
 
 namespace ws {
 
 namespace {
+
+using fp64::divide;
+using fp64::root;
 
 constexpr int BS = 256;
 
@@ -27,32 +31,41 @@ __device__ __forceinline__ void cons_to_prim(int ndim, const double* U, double* 
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (d < ndim) {
-      double u = U[1 + d] / rho;
+      double u = divide(U[1 + d], rho);
       q[1 + d] = u;
       usq = usq + u * u;
     }
   }
   double ke = (0.5 * rho) * usq;
   double E = U[1 + ndim], Gam = U[2 + ndim], Pi = U[3 + ndim];
-  q[1 + ndim] = ((E - ke) - Pi) / Gam;
+  q[1 + ndim] = divide((E - ke) - Pi, Gam);
   q[2 + ndim] = Gam;
   q[3 + ndim] = Pi;
 }
 
 __device__ __forceinline__ double sound_speed2(double rho, double p, double Gam, double Pi) {
-  return (((Gam + 1.0) * p) + Pi) / (Gam * rho);
+  return divide(((Gam + 1.0) * p) + Pi, Gam * rho);
 }
 
 __device__ __forceinline__ bool admissible(double rho, double p, double Gam, double Pi) {
   return (rho > 0.0) && (Gam > 0.0) && ((((Gam + 1.0) * p) + Pi) > 0.0);
 }
 
-// padded coordinates of linear index i
-__device__ __forceinline__ void coords(const GridDev& g, int64_t i, int64_t c[3]) {
-  c[0] = i % g.P[0];
-  int64_t r = i / g.P[0];
-  c[1] = r % g.P[1];
-  c[2] = r / g.P[1];
+// coordinates of linear index i in extents e0, e1 (x fastest), in 32-bit
+// arithmetic where the index allows (a 64-bit division takes about 70
+// instructions)
+__device__ __forceinline__ void coords(int64_t i, int64_t e0, int64_t e1, int64_t c[3]) {
+  if (i < (1LL << 31)) {
+    const unsigned u = (unsigned)i, r = u / (unsigned)e0, z = r / (unsigned)e1;
+    c[0] = u - r * (unsigned)e0;
+    c[1] = r - z * (unsigned)e1;
+    c[2] = z;
+  } else {
+    c[0] = i % e0;
+    const int64_t r = i / e0;
+    c[1] = r % e1;
+    c[2] = r / e1;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -90,24 +103,81 @@ __global__ void k_ghost(GridDev g, double* __restrict__ U, int d) {
   }
 }
 
-// primitives + sound speed of every cell the sweeps read (at most one
-// coordinate outside the interior)
-__global__ void k_prim(GridDev g, const double* __restrict__ U, double* __restrict__ Q) {
+// atomicMax of the threads' values
+__device__ __forceinline__ void block_max(unsigned long long b, unsigned long long* out) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
+    b = v > b ? v : b;
+  }
+  __shared__ unsigned long long sm[32];
+  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (lane == 0) sm[w] = b;
+  __syncthreads();
+  if (w == 0) {
+    b = lane < (int)(blockDim.x >> 5) ? sm[lane] : 0ULL;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
+      b = v > b ? v : b;
+    }
+    if (lane == 0) atomicMax(out, b);
+  }
+}
+
+// The start of an RHS evaluation in one launch: ghost layers of U (of the
+// cells with one coordinate outside the interior: the others are never read),
+// primitives and sound speed of every cell the sweeps read and, with lmax,
+// the CFL rate: max over the interior cells of sum_d (|u_d| + c)/dx_d.
+// Non-negative doubles order like their bit patterns, so the maximum is an
+// integer atomicMax; a NaN orders above +inf.  clear: a counter set to zero.
+template <int NDIM>
+__global__ void __launch_bounds__(BS) k_prep(const __grid_constant__ GridDev g, double* U, double* __restrict__ Q,
+                                             unsigned long long* lmax, unsigned long long* clear) {
+  constexpr int NV = NDIM + 4;
+  if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0ULL;
+  unsigned long long best = 0ULL;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.N; i += (int64_t)gridDim.x * blockDim.x) {
     int64_t c[3];
-    coords(g, i, c);
-    int out = 0;
+    coords(i, g.P[0], g.P[1], c);
+    int out = 0, flip = -1;
+    int64_t src = i;
 #pragma unroll
-    for (int d = 0; d < 3; ++d)
-      if (d < g.ndim && (c[d] < NG || c[d] >= NG + g.n[d])) ++out;
+    for (int d = 0; d < NDIM; ++d) {
+      const int64_t x = c[d] - NG;
+      if (x >= 0 && x < g.n[d]) continue;
+      ++out;
+      const int kind = g.bc[d][x < 0 ? 0 : 1];
+      int64_t m = x < 0 ? 0 : g.n[d] - 1;
+      if (kind == WS_BC_PERIODIC) m = x < 0 ? x + g.n[d] : x - g.n[d];
+      if (kind == WS_BC_REFLECTIVE) {
+        m = x < 0 ? -1 - x : 2 * (int64_t)g.n[d] - 1 - x;
+        flip = 1 + d;
+      }
+      src += (m - x) * g.st[d];
+    }
     if (out > 1) continue;
-    double u[MAXV], q[MAXV];
-    for (int f = 0; f < g.nv; ++f) u[f] = U[f * g.N + i];
-    cons_to_prim(g.ndim, u, q);
-    for (int f = 0; f < g.nv; ++f) Q[f * g.N + i] = q[f];
-    int nd = g.ndim;
-    Q[g.nv * g.N + i] = sqrt(sound_speed2(q[0], q[1 + nd], q[2 + nd], q[3 + nd]));
+    double u[NV], q[NV];
+#pragma unroll
+    for (int f = 0; f < NV; ++f) {
+      u[f] = U[f * g.N + src];
+      if (f == flip) u[f] = -u[f];
+      if (out) U[f * g.N + i] = u[f];
+    }
+    cons_to_prim(NDIM, u, q);
+    const double cs = root(sound_speed2(q[0], q[1 + NDIM], q[2 + NDIM], q[3 + NDIM]));
+#pragma unroll
+    for (int f = 0; f < NV; ++f) Q[f * g.N + i] = q[f];
+    Q[NV * g.N + i] = cs;
+    if (lmax && !out) {
+      double lam = 0.0;
+#pragma unroll
+      for (int d = 0; d < NDIM; ++d) lam = lam + divide(fabs(q[1 + d]) + cs, g.dx[d]);
+      const unsigned long long b = lam <= 0.0 ? 0ULL : (unsigned long long)__double_as_longlong(lam);
+      best = b > best ? b : best;
+    }
   }
+  if (lmax) block_max(best, lmax);
 }
 
 __global__ void k_prim_to_cons(GridDev g, const double* __restrict__ Q, double* __restrict__ U) {
@@ -138,43 +208,6 @@ __global__ void k_cons_to_prim_all(GridDev g, const double* __restrict__ U, doub
   }
 }
 
-// max over interior cells of sum_d (|u_d| + c)/dx_d; non-negative doubles
-// order like their bit patterns, so the max is an integer atomicMax.
-__global__ void k_cfl(GridDev g, const double* __restrict__ Q, unsigned long long* lmax) {
-  double best = 0.0;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < g.ncell; t += (int64_t)gridDim.x * blockDim.x) {
-    int64_t x = t % g.n[0];
-    int64_t r = t / g.n[0];
-    int64_t y = r % g.n[1];
-    int64_t z = r / g.n[1];
-    int64_t i = (g.G[0] + x) * g.st[0] + (g.G[1] + y) * g.st[1] + (g.G[2] + z) * g.st[2];
-    double c = Q[g.nv * g.N + i];
-    double lam = 0.0;
-    for (int d = 0; d < g.ndim; ++d) lam = lam + (fabs(Q[(1 + d) * g.N + i]) + c) / g.dx[d];
-    // NaN propagates (it orders above +inf as bits)
-    if (!(lam <= best)) best = lam;
-  }
-  unsigned long long b = (unsigned long long)__double_as_longlong(best);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
-    b = v > b ? v : b;
-  }
-  __shared__ unsigned long long sm[32];
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) sm[w] = b;
-  __syncthreads();
-  if (w == 0) {
-    b = lane < (int)(blockDim.x >> 5) ? sm[lane] : 0ULL;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
-      b = v > b ? v : b;
-    }
-    if (lane == 0) atomicMax(lmax, b);
-  }
-}
-
 __global__ void k_set_dt(double dt_fixed, double cfl, const unsigned long long* __restrict__ lmax,
                          double* __restrict__ dt, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -186,63 +219,80 @@ __global__ void k_set_dt(double dt_fixed, double cfl, const unsigned long long* 
 }
 
 // Sec. 3.1: L(U) summed over x, y, z, then the SSP-RK3 stage.
-// stage -1: write L itself; 0, 1, 2: the three Shu-Osher stages.  Uout may
-// alias Un or Us (each thread reads its cell before writing it).
-template <typename FT>
-__global__ void k_update(GridDev g, int stage, const double* Un, const double* Us, double* Uout, const FT* __restrict__ F0, const FT* __restrict__ F1,
-                         const FT* __restrict__ F2, const FT* __restrict__ u0, const FT* __restrict__ u1,
-                         const FT* __restrict__ u2, const double* __restrict__ dtp, unsigned long long* nbad) {
-  const FT* Fd[3] = {F0, F1, F2};
-  const FT* ud[3] = {u0, u1, u2};
+// stage -1: write L itself; 0, 1, 2: the three Shu-Osher stages.  Stage 0
+// derives the step (dt_fixed, or cfl / *lmax) and leaves it in *dtp for the
+// others.  Uout may alias Un or Us (each thread reads its cell before writing
+// it).
+struct UpdateArgs {
+  GridDev g;
+  int stage;
+  const double *Un, *Us;
+  double* Uout;
+  const double* F[3];
+  const double* u[3];
+  double dt_fixed, cfl;
+  const unsigned long long* lmax;
+  double* dtp;
+  unsigned long long* nbad;
+};
+
+template <int NDIM>
+__global__ void __launch_bounds__(BS) k_update(const __grid_constant__ UpdateArgs a) {
+  constexpr int NV = NDIM + 4;
+  const GridDev& g = a.g;
   const double c13 = 1.0 / 3.0, c23 = 2.0 / 3.0;
+  double dt = 0.0;
+  if (a.stage == 0) {
+    dt = a.dt_fixed > 0.0 ? a.dt_fixed : divide(a.cfl, __longlong_as_double((long long)*a.lmax));
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.dtp = dt;
+  } else if (a.stage > 0) {
+    dt = *a.dtp;
+  }
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < g.ncell; t += (int64_t)gridDim.x * blockDim.x) {
-    int64_t a[3];
-    a[0] = t % g.n[0];
-    int64_t r = t / g.n[0];
-    a[1] = r % g.n[1];
-    a[2] = r / g.n[1];
-    int64_t i = (g.G[0] + a[0]) * g.st[0] + (g.G[1] + a[1]) * g.st[1] + (g.G[2] + a[2]) * g.st[2];
-    int64_t fl[3], fr[3];
-    double du[3];
-    for (int d = 0; d < g.ndim; ++d) {
-      int64_t b[3] = {a[0], a[1], a[2]};
-      fl[d] = (b[2] * g.fe[d][1] + b[1]) * g.fe[d][0] + b[0];
-      b[d] += 1;
-      fr[d] = (b[2] * g.fe[d][1] + b[1]) * g.fe[d][0] + b[0];
-      du[d] = (double)ud[d][fr[d]] - (double)ud[d][fl[d]];
+    int64_t c[3];
+    coords(t, g.n[0], g.n[1], c);
+    const int64_t i = (g.G[0] + c[0]) * g.st[0] + (g.G[1] + c[1]) * g.st[1] + (g.G[2] + c[2]) * g.st[2];
+    int64_t fl[NDIM], fr[NDIM];
+    double du[NDIM];
+#pragma unroll
+    for (int d = 0; d < NDIM; ++d) {
+      fl[d] = (c[2] * g.fe[d][1] + c[1]) * g.fe[d][0] + c[0];
+      fr[d] = fl[d] + (d == 0 ? 1 : (d == 1 ? g.fe[d][0] : g.fe[d][0] * g.fe[d][1]));
+      du[d] = divide(a.u[d][fr[d]] - a.u[d][fl[d]], g.dx[d]);
     }
-    double dt = stage >= 0 ? dtp[0] : 0.0;
-    double out[MAXV];
-    for (int f = 0; f < g.nv; ++f) {
+    double out[NV];
+#pragma unroll
+    for (int f = 0; f < NV; ++f) {
       double L = 0.0;
-      double phi = Us[f * g.N + i];
-      for (int d = 0; d < g.ndim; ++d) {
-        int64_t nf = g.nfaces[d];
-        double dF = (double)Fd[d][f * nf + fr[d]] - (double)Fd[d][f * nf + fl[d]];
-        double term = -(dF / g.dx[d]);
-        if (f >= 2 + g.ndim) term = term + phi * (du[d] / g.dx[d]);
+      const double phi = a.Us[f * g.N + i];
+#pragma unroll
+      for (int d = 0; d < NDIM; ++d) {
+        const int64_t nf = g.nfaces[d];
+        const double dF = a.F[d][f * nf + fr[d]] - a.F[d][f * nf + fl[d]];
+        double term = -divide(dF, g.dx[d]);
+        if (f >= 2 + NDIM) term = term + phi * du[d];
         L = L + term;
       }
       double o;
-      if (stage < 0) {
+      if (a.stage < 0) {
         o = L;
       } else {
-        double un = Un[f * g.N + i];
-        if (stage == 0)
+        const double un = a.Un[f * g.N + i];
+        if (a.stage == 0)
           o = un + dt * L;
-        else if (stage == 1)
+        else if (a.stage == 1)
           o = (0.75 * un) + (0.25 * (phi + dt * L));
         else
           o = (c13 * un) + (c23 * (phi + dt * L));
       }
       out[f] = o;
     }
-    for (int f = 0; f < g.nv; ++f) Uout[f * g.N + i] = out[f];
-    if (stage == 2) {
-      double q[MAXV];
-      cons_to_prim(g.ndim, out, q);
-      int nd = g.ndim;
-      if (!admissible(q[0], q[1 + nd], q[2 + nd], q[3 + nd])) atomicAdd(nbad, 1ULL);
+#pragma unroll
+    for (int f = 0; f < NV; ++f) a.Uout[f * g.N + i] = out[f];
+    if (a.stage == 2) {
+      double q[NV];
+      cons_to_prim(NDIM, out, q);
+      if (!admissible(q[0], q[1 + NDIM], q[2 + NDIM], q[3 + NDIM])) atomicAdd(a.nbad, 1ULL);
     }
   }
 }
@@ -278,8 +328,14 @@ void launch_ghost(const GridDev& g, double* U, int d, cudaStream_t s) {
   k_ghost<<<blocks_for(total), BS, 0, s>>>(g, U, d);
 }
 
-void launch_prim(const GridDev& g, const double* U, double* Q, cudaStream_t s) {
-  k_prim<<<blocks_for(g.N), BS, 0, s>>>(g, U, Q);
+void launch_prep(const GridDev& g, double* U, double* Q, unsigned long long* lmax, unsigned long long* clear,
+                 cudaStream_t s) {
+  const int b = blocks_for(g.N);
+  switch (g.ndim) {
+    case 1: k_prep<1><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
+    case 2: k_prep<2><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
+    default: k_prep<3><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
+  }
 }
 
 void launch_prim_to_cons(const GridDev& g, const double* Q, double* U, cudaStream_t s) {
@@ -290,22 +346,21 @@ void launch_cons_to_prim_all(const GridDev& g, const double* U, double* Q, cudaS
   k_cons_to_prim_all<<<blocks_for(g.N), BS, 0, s>>>(g, U, Q);
 }
 
-void launch_cfl(const GridDev& g, const double* Q, unsigned long long* lmax, cudaStream_t s) {
-  int b = blocks_for(g.ncell);
-  if (b > 152 * 8) b = 152 * 8;
-  k_cfl<<<b, BS, 0, s>>>(g, Q, lmax);
-}
-
 void launch_set_dt(const double*, double dt_fixed, double cfl, const unsigned long long* lmax, double* dt_dev,
                    int64_t n, cudaStream_t s) {
   k_set_dt<<<blocks_for(n), BS, 0, s>>>(dt_fixed, cfl, lmax, dt_dev, n);
 }
 
 void launch_update(const GridDev& g, int stage, const double* Un, const double* Us, double* Uout,
-                   double* const Fh[3], double* const us[3], const double* dt_dev, unsigned long long* nbad,
-                   cudaStream_t s) {
-  k_update<double><<<blocks_for(g.ncell), BS, 0, s>>>(g, stage, Un, Us, Uout, Fh[0], Fh[1], Fh[2], us[0], us[1],
-                                                      us[2], dt_dev, nbad);
+                   double* const Fh[3], double* const us[3], double dt_fixed, double cfl,
+                   const unsigned long long* lmax, double* dt_dev, unsigned long long* nbad, cudaStream_t s) {
+  UpdateArgs a{g, stage, Un, Us, Uout, {Fh[0], Fh[1], Fh[2]}, {us[0], us[1], us[2]}, dt_fixed, cfl, lmax, dt_dev, nbad};
+  const int b = blocks_for(g.ncell);
+  switch (g.ndim) {
+    case 1: k_update<1><<<b, BS, 0, s>>>(a); break;
+    case 2: k_update<2><<<b, BS, 0, s>>>(a); break;
+    default: k_update<3><<<b, BS, 0, s>>>(a); break;
+  }
 }
 
 void launch_mood_count(const uint8_t* mask, int64_t n, int64_t nstage, const int64_t* dir_off, int ndim,

@@ -142,21 +142,24 @@ namespace ws {
 
 // ---- launchers (ws_common.cu, built with -fmad=false) ----
 void launch_ghost(const GridDev& g, double* U, int d, cudaStream_t s);
-void launch_prim(const GridDev& g, const double* U, double* Q, cudaStream_t s);
+// ghost layers of U, primitives Q and (lmax non-null, zeroed before) the CFL
+// rate; clear (nullable): a counter the launch sets to zero
+void launch_prep(const GridDev& g, double* U, double* Q, unsigned long long* lmax, unsigned long long* clear,
+                 cudaStream_t s);
 void launch_prim_to_cons(const GridDev& g, const double* Q, double* U, cudaStream_t s);
 void launch_cons_to_prim_all(const GridDev& g, const double* U, double* Q, cudaStream_t s);
-void launch_cfl(const GridDev& g, const double* Q, unsigned long long* lmax, cudaStream_t s);
 void launch_set_dt(const double* dt_fixed_or_null, double dt_fixed, double cfl, const unsigned long long* lmax,
                    double* dt_dev, int64_t n, cudaStream_t s);
 void launch_update(const GridDev& g, int stage, const double* Un, const double* Us, double* Uout,
-                   double* const Fh[3], double* const us[3], const double* dt_dev, unsigned long long* nbad,
-                   cudaStream_t s);
+                   double* const Fh[3], double* const us[3], double dt_fixed, double cfl,
+                   const unsigned long long* lmax, double* dt_dev, unsigned long long* nbad, cudaStream_t s);
 void launch_mood_count(const uint8_t* mask, int64_t n, int64_t nstage, const int64_t* dir_off, int ndim,
                        unsigned long long* counts, cudaStream_t s);
 
 // ---- FP64 sweep (ws_fp64.cu, built with -fmad=false) ----
-void launch_face_fp64(const GridDev& g, int d, const double* Q, double* Fh, double* us, uint8_t* mask,
-                      double eps, int mood, int weights, cudaStream_t s);
+// the faces of all directions (mask: nullable, as a whole or per direction)
+void launch_face_fp64(const GridDev& g, const double* Q, double* const Fh[3], double* const us[3],
+                      uint8_t* const mask[3], double eps, int mood, int weights, cudaStream_t s);
 
 // ---- mixed-precision sweep (ws_mixed.cu, FMA allowed) ----
 void launch_prim32(const GridDev& g, const double* U, float* Q, cudaStream_t s);

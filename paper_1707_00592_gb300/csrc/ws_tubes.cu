@@ -41,18 +41,18 @@ __global__ void k_tubes_prim(TubesDev t, const double* __restrict__ U, double* _
   const int64_t N = t.total;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
     double rho = U[i];
-    double u = U[N + i] / rho;
+    double u = divide(U[N + i], rho);
     double usq = 0.0;
     usq = usq + u * u;
     double ke = (0.5 * rho) * usq;
     double E = U[2 * N + i], Gam = U[3 * N + i], Pi = U[4 * N + i];
-    double p = ((E - ke) - Pi) / Gam;
+    double p = divide((E - ke) - Pi, Gam);
     Q[i] = rho;
     Q[N + i] = u;
     Q[2 * N + i] = p;
     Q[3 * N + i] = Gam;
     Q[4 * N + i] = Pi;
-    Q[5 * N + i] = sqrt(sound_speed2(rho, p, Gam, Pi));
+    Q[5 * N + i] = root(sound_speed2(rho, p, Gam, Pi));
   }
 }
 
@@ -67,9 +67,9 @@ __global__ void k_tubes_cfl(TubesDev t, const double* __restrict__ Q, unsigned l
       tube = t.cell_tube[i];
       int64_t a = t.off[tube], e = t.off[tube + 1];
       if (i >= a + NG && i < e - NG) {
-        double dx = 1.0 / (double)(e - a - 2 * NG);
+        const double dx = divide(1.0, (double)(e - a - 2 * NG));
         double lam = 0.0;
-        lam = lam + (fabs(Q[N + i]) + Q[5 * N + i]) / dx;
+        lam = lam + divide(fabs(Q[N + i]) + Q[5 * N + i], dx);
         b = (unsigned long long)__double_as_longlong(lam);
       }
     }
@@ -90,35 +90,58 @@ __global__ void k_tubes_cfl(TubesDev t, const double* __restrict__ Q, unsigned l
 }
 
 // face i+1/2 of a tube stored at padded cell i (faces -1/2 .. len-1/2 sit on
-// the cells off+2 .. off+len+2); other cells get the mask byte 0xff.
-template <bool JS>
-__global__ void __launch_bounds__(128) k_tubes_face(TubesDev t, const double* __restrict__ Q, double* __restrict__ Fh,
+// the cells off+2 .. off+len+2); other cells get the mask byte 0xff.  One CTA:
+// CH chunks of FPW consecutive padded cells.
+template <int CH, Scheme SC, int PI>
+__global__ void __launch_bounds__(160) k_tubes_face(TubesDev t, const double* __restrict__ Q, double* __restrict__ Fh,
                                                     double* __restrict__ us, uint8_t* __restrict__ mask, double eps,
                                                     int mood, int weights) {
+  constexpr int H = 3;
+  __shared__ FaceSmem<5, CH> sm;
   const int64_t N = t.total;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    int tube = t.cell_tube[i];
-    int64_t a = t.off[tube], e = t.off[tube + 1];
-    if (i < a + NG - 1 || i > e - NG - 1) {
-      if (mask) mask[i] = 0xff;
-      continue;
+  const int lane = threadIdx.x & 31, side = lane & 1;
+  const int64_t i0 = blockIdx.x * (int64_t)(CH * FPW) + (lane >> 1);
+  // the face of cell i, or the tube's nearest one where cell i carries none
+  auto face_cell = [&](int64_t i) {
+    const int tube = t.cell_tube[i < N ? i : N - 1];
+    const int64_t lo = t.off[tube] + NG - 1, hi = t.off[tube + 1] - NG - 1;
+    return i < lo ? lo : (i > hi ? hi : i);
+  };
+  auto at = [&](int k) {
+    Faces<5> fc;
+    fc.q = Q;
+    fc.N = N;
+    fc.d = 0;
+    fc.st = 1;
+    fc.base = face_cell(i0 + k * FPW) - 2;
+    return fc;
+  };
+  cta_faces<5, CH, SC, PI>(sm, eps, mood, weights, at, [&](int k, const Faces<5>& fc, const double (&out)[H], int code) {
+    const int other = __shfl_xor_sync(ALL, code, 1);
+    const int64_t i = i0 + k * FPW;
+    if (i >= N) return;
+    const bool live = fc.base + 2 == i;
+    if (mask && side == 0) mask[i] = live ? (uint8_t)(code | (other << 2)) : 0xff;
+    if (!live) return;
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      const int m = (side ? H : 0) + j;
+      if (m < 5)
+        Fh[m * N + i] = out[j];
+      else
+        us[i] = out[j];
     }
-    double qc[6][5], cc[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      int64_t idx = i + (j - 2);
-#pragma unroll
-      for (int m = 0; m < 5; ++m) qc[j][m] = Q[m * N + idx];
-      cc[j] = Q[5 * N + idx];
-    }
-    double Fhat[5], ustar;
-    int cl, cr;
-    face<5, JS>(qc, cc, eps, mood, weights, Fhat, ustar, cl, cr);
-#pragma unroll
-    for (int m = 0; m < 5; ++m) Fh[m * N + i] = Fhat[m];
-    us[i] = ustar;
-    if (mask) mask[i] = (uint8_t)(cl | (cr << 2));
-  }
+  });
+}
+
+template <Scheme SC>
+void tubes_face(const TubesDev& t, const double* Q, double* Fh, double* us, uint8_t* mask, double eps, int mood,
+                int weights, cudaStream_t s) {
+  const unsigned b = (unsigned)((t.total + 5 * FPW - 1) / (5 * FPW)), b1 = (unsigned)((t.total + FPW - 1) / FPW);
+  if (SC != LITERAL && large_sweep(b))
+    k_tubes_face<5, SC, PIPES><<<b, 160, 0, s>>>(t, Q, Fh, us, mask, eps, mood, weights);
+  else
+    k_tubes_face<1, SC, CHAIN><<<b1, 160, 0, s>>>(t, Q, Fh, us, mask, eps, mood, weights);
 }
 
 __global__ void k_tubes_update(TubesDev t, int stage, const double* Un, const double* Us, double* Uout,
@@ -130,16 +153,16 @@ __global__ void k_tubes_update(TubesDev t, int stage, const double* Un, const do
     int tube = t.cell_tube[i];
     int64_t a = t.off[tube], e = t.off[tube + 1];
     if (i < a + NG || i >= e - NG) continue;
-    double dx = 1.0 / (double)(e - a - 2 * NG);
+    const double dx = divide(1.0, (double)(e - a - 2 * NG));
     double dt = dtp[tube];
-    double du = us[i] - us[i - 1];
+    const double dudx = divide(us[i] - us[i - 1], dx);
     double out[5];
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
       double phi = Us[f * N + i];
       double dF = Fh[f * N + i] - Fh[f * N + i - 1];
-      double term = -(dF / dx);
-      if (f >= 3) term = term + phi * (du / dx);
+      double term = -divide(dF, dx);
+      if (f >= 3) term = term + phi * dudx;
       double L = 0.0;
       L = L + term;
       double un = Un[f * N + i];
@@ -156,10 +179,10 @@ __global__ void k_tubes_update(TubesDev t, int stage, const double* Un, const do
     for (int f = 0; f < 5; ++f) Uout[f * N + i] = out[f];
     if (stage == 2) {
       double rho = out[0];
-      double u = out[1] / rho;
+      double u = divide(out[1], rho);
       double usq = 0.0;
       usq = usq + u * u;
-      double p = ((out[2] - (0.5 * rho) * usq) - out[4]) / out[3];
+      double p = divide((out[2] - (0.5 * rho) * usq) - out[4], out[3]);
       bool ok = (rho > 0.0) && (out[3] > 0.0) && ((((out[3] + 1.0) * p) + out[4]) > 0.0);
       if (!ok) atomicAdd(nbad, 1ULL);
     }
@@ -179,10 +202,11 @@ void launch_tubes_cfl(const TubesDev& t, const double* Q, unsigned long long* lm
 }
 void launch_tubes_face_fp64(const TubesDev& t, const double* Q, double* Fh, double* us, uint8_t* mask, double eps,
                             int mood, int weights, cudaStream_t s) {
-  if (weights == WS_W_JS)
-    k_tubes_face<true><<<blocks_for(t.total, 128), 128, 0, s>>>(t, Q, Fh, us, mask, eps, mood, weights);
-  else
-    k_tubes_face<false><<<blocks_for(t.total, 128), 128, 0, s>>>(t, Q, Fh, us, mask, eps, mood, weights);
+  switch (scheme_of(eps, weights)) {
+    case JS: tubes_face<JS>(t, Q, Fh, us, mask, eps, mood, weights, s); break;
+    case LITERAL: tubes_face<LITERAL>(t, Q, Fh, us, mask, eps, mood, weights, s); break;
+    default: tubes_face<IS>(t, Q, Fh, us, mask, eps, mood, weights, s);
+  }
 }
 void launch_tubes_update(const TubesDev& t, int stage, const double* Un, const double* Us, double* Uout,
                          const double* Fh, const double* us, const double* dt_dev, unsigned long long* nbad,

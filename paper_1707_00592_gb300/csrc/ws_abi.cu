@@ -120,6 +120,7 @@ void free_all(ws_ctx* c) {
   cudaFree(c->Q);
   cudaFree(c->Q32);
   cudaFree(c->chain);
+  cudaFree(c->moving);
   cudaFree(c->img[0]);
   cudaFree(c->img[1]);
   cudaFree(c->Ka);
@@ -307,6 +308,12 @@ int fused_run3(ws_ctx* c, double* U, double dt, const GateArgs* gate, const int*
   } else {
     c->img_cur = -1;
   }
+  // a captured step would replay one stamp
+  int* moving = one_scope && !c->capturing ? c->moving : nullptr;
+  if (moving && ++c->stamp == 0x7fffffff) {  // the stamps start over
+    CK(c, cudaMemsetAsync(moving, 0, 2 * sizeof(int) * fused2d_max_tiles(g), c->stream));
+    c->stamp = 1;
+  }
   for (int s = 0; s < 3; ++s) {
     uint8_t* mb = c->mask + (int64_t)s * c->nmask;
     std::optional<KScope> k;
@@ -328,7 +335,7 @@ int fused_run3(ws_ctx* c, double* U, double dt, const GateArgs* gate, const int*
                      mb + c->mask_off[1], (float)c->opts.eps, c->opts.mood, c->opts.weights, nbad, gate, run_if,
                      census, c->stage_tile, c->stage_sched == 0, s == 0 && img_in, s == 2 ? img_out : nullptr, tmk,
                      tmv, s == 2 ? clr0 : nullptr, s == 2 ? clr1 : nullptr, c->tail_rows, map2_of(c, tmk),
-                     map2_of(c, tmv), c->stream);
+                     map2_of(c, tmv), moving, c->stamp, c->stream);
     }
   }
   return check_launch(c, "fused stage");
@@ -525,8 +532,12 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
       if ((rc = dalloc(c, &c->Q32, std::max((int64_t)(g.nv + 1) * g.N, (int64_t)g.nv * g.N32)))) goto bad;
       if (fused2d) {
         if ((rc = dalloc(c, &c->Ka, (int64_t)g.nv * g.N32)) || (rc = dalloc(c, &c->Kb, (int64_t)g.nv * g.N32)) ||
-            (rc = dalloc(c, &c->census, 4)))
+            (rc = dalloc(c, &c->census, 4)) || (rc = dalloc(c, &c->moving, 2 * fused2d_max_tiles(g))))
           goto bad;
+        if (cudaMemset(c->moving, 0, 2 * sizeof(int) * fused2d_max_tiles(g)) != cudaSuccess) {
+          rc = fail(c, WS_ECUDA, "cannot clear the tile marks");
+          goto bad;
+        }
         if (fused2d_prepare() != cudaSuccess) {
           rc = fail(c, WS_ECUDA, "cannot enable %d bytes of shared memory for the fused stage", fused2d_smem_bytes());
           goto bad;
@@ -1130,7 +1141,7 @@ int ws_gate_eval(ws_ctx* c, double* U, uint8_t* smooth) {
   launch_stage2d(c->gd, 3, U, c->Q32, c->Ka, c->Kb, 0.0, c->opts.cfl, c->lmax, c->dt_dev, smooth,
                  smooth + c->mask_off[1], (float)c->opts.eps, c->opts.mood, c->opts.weights, c->nbad, &ga, nullptr,
                  nullptr, 0, false, false, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr,
-                 c->stream);
+                 nullptr, 0, c->stream);
   return check_launch(c, "gate eval");
 }
 

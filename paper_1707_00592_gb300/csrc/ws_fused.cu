@@ -28,7 +28,8 @@
 // evaluated in this launch, or decisions stored by an earlier stage of the
 // step); 3 the census: the plain stage, bit for bit, that also counts per
 // face-variable whether the stencil was flat (linear weights) or took
-// WENO-IS, and per warp whether the WENO-IS branch ran.
+// WENO-IS, and per warp whether the WENO-IS branch ran; 4 the plain 2D stage
+// that takes quiet tiles the short way (see quiet_state).
 //
 // The Shu-Osher SSP-RK3 is carried in increment form, algebraically
 // identical to U1 = U + dt L0, U2 = 3/4 U + 1/4 (U1 + dt L1),
@@ -156,13 +157,14 @@ struct Smem {
   unsigned long long red[NT / 32];  // per-warp CFL maxima
   unsigned long long mbar;          // completion of the TMA loads
   float dt;                         // the step, broadcast from thread 0
+  int moved[5];                     // quiet tiles: marks of this tile and its neighbours
 };
 
 // Two 2D stage CTAs of the default tile, with the 1 KiB the hardware keeps
 // per CTA, fit the 196 KiB shared-memory carveout of an SM: the next larger
 // carveout would leave the halo loads of boundary tiles 28 KiB of L1 instead
 // of 60 (measured: 10 % slower per-thread loads).
-static_assert(2 * (sizeof(Smem<0, 6, 0, Tile<32, 15, 512>>) + 1024) <= 196 * 1024,
+static_assert(2 * (sizeof(Smem<4, 6, 0, Tile<32, 15, 512>>) + 1024) <= 196 * 1024,
               "the default 2D stage no longer leaves room for L1");
 // The 3D passes keep their CTAs per SM: four of 32 x 7 cells, two of 32 x 15
 // (228 KiB of shared memory per SM at most).
@@ -229,6 +231,11 @@ struct StageArgs {
   int rows_full;
   alignas(64) CUtensorMap tm_k2;
   alignas(64) CUtensorMap tm_v2;
+  // Quiet tiles (GATE 4): per tile, the stamp of the last step in which it was
+  // not quiet in stage 0, 1
+  int* moving0;
+  int* moving1;
+  int stamp;
   // nullable: slots block (0, 0, 0) clears once the previous grid has
   // completed (a step's last launch clears the next step's CFL maximum and
   // inadmissible-cell count, so consecutive steps need no memset between them)
@@ -553,6 +560,31 @@ __device__ __forceinline__ bool mbar_wait0(unsigned long long* bar, unsigned lon
   }
 }
 
+// Quiet tiles.  Where all cells of a tile and its halo hold one state (fluid
+// that no wave has reached: a sixth of the tiles over a shock-bubble run, a
+// third or more over a shock-cylinder run), all faces of a direction carry one
+// flux and the divergence is zero.  Stage 0 finds these tiles, at no cost in
+// synchronisation: a warp that holds two different states marks the tile as
+// moving.  A tile with only quiet tiles beside it then has the same uniform
+// state in stage 1, and likewise in stage 2: it writes its zero increments
+// and MOOD bytes and is done, with the bits that the evaluation would give.  (A
+// barrier in stage 0 that told every tile whether it is quiet cost the moving
+// ones 2 to 3 %.)
+// The neighbours must hold the halo: callers pass no marks when a periodic
+// axis ends in a tile of less than three cells.
+//
+// The reconstruction of a uniform state is that state to a few ulps.  With
+// the margin tested here it is admissible at 5th order (MOOD byte 0) and its
+// flux is finite.
+template <class T>
+__device__ __forceinline__ bool quiet_state(const float* r) {  // a cell of the q tile
+  constexpr int FS = T::FS;
+  const float rho = r[0], p = r[T::IP * FS], G = r[T::IG * FS], Pi = r[T::IPI * FS], c = r[T::IC * FS];
+  const float un = fabsf(r[FS]) + fabsf(r[2 * FS]);
+  return rho > 1e-20f && rho < 1e20f && G > 1e-6f && G < 1e6f && c > 1e-6f && un + c < 1e9f && fabsf(p) < 1e18f &&
+         fabsf(Pi) < 1e18f && fmaf(G + 1.0f, p, Pi) > 1e-4f * ((G + 1.0f) * (fabsf(p) + rho * c * un) + fabsf(Pi));
+}
+
 // One CTA's work: the tile in tile row `trow` of tiles TL starting at grid row
 // `ybase`.  MAP 1 takes the second pair of TMA descriptors (boxes of TL).
 template <int GATE, int NQ_, int MODE, class TL, int MAP>
@@ -562,6 +594,7 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
   constexpr int TX = TL::TX, TY = TL::TY, NT = TL::NT, NF = TL::NF, NMT = TL::NMT;
   constexpr bool LEARNED = GATE == 1 || GATE == 2;  // faces may take the linear weights by the gate's decision
   constexpr bool CENSUS = GATE == 3;
+  constexpr bool QUIET = GATE == 4;  // looks for quiet tiles
   constexpr int NQ = NQ_, ND = T::ND, FS = T::FS;
   constexpr bool CACHE = SM::CACHE;
   // axes: x, the tile's 2nd axis (y; z in pass 2), the plane axis (z; y in pass 2; none in 2D)
@@ -632,6 +665,21 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
       if (a.stage != 0) tma_load_4d(&S.kbox[0][0][0], &a.tm_k, x0, g.G[1] + plane, y0, 0, &S.mbar);
     }
   }
+  const int tile_id = blockIdx.y * gridDim.x + blockIdx.x;
+  if constexpr (QUIET) {
+    // The marks of this tile and, in stages 1 and 2, of its four neighbours,
+    // copied by a warp of its own (thread 0 has the step and the boxes to wait
+    // for) and asynchronously (a load would hold up its share of phase A).
+    if (tid >= 32 && tid < 37) {
+      const int W = gridDim.x, H = gridDim.y, bx = blockIdx.x, by = blockIdx.y;
+      int tx = bx + (tid == 33 ? -1 : (tid == 34 ? 1 : 0)), ty = by + (tid == 35 ? -1 : (tid == 36 ? 1 : 0));
+      if (tx < 0 || tx >= W) tx = g.bc[0][0] == WS_BC_PERIODIC ? (tx < 0 ? W - 1 : 0) : bx;
+      if (ty < 0 || ty >= H) ty = g.bc[1][0] == WS_BC_PERIODIC ? (ty < 0 ? H - 1 : 0) : by;
+      if (a.stage != 0 || tid == 32) cp_async4(&S.moved[tid - 32], &(a.stage == 2 ? a.moving1 : a.moving0)[ty * W + tx]);
+      cp_async_commit();
+      if (a.stage != 0) cp_async_wait_all();
+    }
+  }
   if (a.stage == 1 || a.stage == 2 || tma) {
     if (tid == 0) {
       if (a.stage == 1 || a.stage == 2) {  // one FP64 division per CTA
@@ -646,6 +694,45 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
       if (tma && !mbar_wait0(&S.mbar, 1000000000ULL)) atomicAdd(a.nbad, 1ULL << 40);
     }
     __syncthreads();
+  }
+  // the end of a quiet tile: its increments (stages 0, 1) or the image of its
+  // state (stage 2), and MOOD bytes
+  auto quiet_end = [&]() {
+    float* out = a.stage == 0 || a.stage == 1 ? a.Kout : a.img_out;
+    if (out) {
+      float v[NQ];
+#pragma unroll
+      for (int m = 0; m < NQ; ++m) v[m] = a.stage == 2 ? a.U32[m * N32 + idx32(y0, x0)] : 0.0f;
+      for (int c = tid; c < TX * TY; c += NT) {
+        const int j = c / TX, i = c - j * TX;
+        if (x0 + i >= nx || y0 + j >= n1) continue;
+        const int64_t gf = idx32(y0 + j, x0 + i);
+#pragma unroll
+        for (int m = 0; m < NQ; ++m) out[m * N32 + gf] = v[m];
+      }
+    }
+    for (int f = tid; f < T::NFP; f += NT) {
+      bool isx;
+      int hx, hy;
+      if (!face_geom<T::XF, TL>(f, x0, y0, nx, n1, isx, hx, hy)) continue;
+      if (isx) {
+        if (a.mask_x) a.mask_x[(int64_t)(y0 + hy - NG) * (nx + 1) + (x0 + hx)] = 0;
+      } else if (a.mask_a) {
+        a.mask_a[(int64_t)(y0 + hy) * nx + (x0 + hx - T::QX)] = 0;
+      }
+    }
+  };
+  if constexpr (QUIET) {
+    if (a.stage != 0) {
+      bool quiet = true;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) quiet = quiet && S.moved[k] != a.stamp;
+      if (quiet) {
+        quiet_end();
+        return;
+      }
+      if (a.stage == 1 && tid == 0) a.moving1[tile_id] = a.stamp;
+    }
   }
   // The own cells' FP64 state (stage 2) and, in the second 3D pass, the x + y
   // part of their divergence are needed only in phase C: they are copied into
@@ -673,6 +760,7 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
   const float dt = (a.stage == 1 || a.stage == 2) ? S.dt : 0.0f;
   const float coef = a.stage == 0 ? 0.0f : (a.stage == 1 ? dt : 0.25f * dt);
   float lam_max = 0.0f;
+  float p_own = -1.0f;  // QUIET, stage 0: a pressure of this thread's cells
 
   if (LEARNED) {  // this thread's drift sums (only it touches them until after phase B)
     SG.dpart[0][tid] = 0.0f;
@@ -721,6 +809,7 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
       float ksq = ND == 2 ? fmaf(vel[0], vel[0], vel[1] * vel[1])
                           : fmaf(vel[0], vel[0], fmaf(vel[1], vel[1], vel[ND - 1] * vel[ND - 1]));
       float p = fmaf(-0.5f * rho, ksq, eint) * frcp(Gam);
+      if (QUIET) p_own = p;
       S.q[0][hy][hx] = rho;
 #pragma unroll
       for (int d = 0; d < ND; ++d) S.q[1 + d][hy][hx] = vel[d];
@@ -862,12 +951,37 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
     }
     if ((tid & 31) == 0) S.red[tid >> 5] = b;
   }
+  if (QUIET && a.stage == 0 && tid == 32) cp_async_wait_all();
   __syncthreads();
   if (a.stage == 0 && MODE != 2 && tid == 0) {
     unsigned long long b = 0;
 #pragma unroll
     for (int w = 0; w < NT / 32; ++w) b = S.red[w] > b ? S.red[w] : b;
     if (b) atomicMax(a.lmax, b);
+  }
+  if constexpr (QUIET) {
+    if (a.stage == 0) {  // mark the tile unless its cells hold one state
+      const float* ref = &S.q[0][NG][T::QX];
+      // most moving tiles show in the pressures alone
+      bool eq = __all_sync(0xffffffffu, p_own == ref[T::IP * FS] || p_own == -1.0f);
+      if (eq) {
+        for (int h = tid; h < T::NH; h += NT) {
+          const int hy = h / T::QW, hx = h - hy * T::QW + T::QL;
+          const int gx = x0 + hx - T::QX, ga = y0 + hy - NG;
+          if ((gx < 0 || gx >= nx) && (ga < 0 || ga >= n1)) continue;  // never filled, never read
+#pragma unroll
+          for (int m = 0; m < NQ; ++m) eq = eq && S.q[m][hy][hx] == ref[m * FS];
+        }
+        eq = __all_sync(0xffffffffu, eq && quiet_state<T>(ref));
+      }
+      // quiet one step ago and now: this stage is done, too (the barrier that
+      // tells is not worth its wait in the other tiles)
+      if (S.moved[0] != a.stamp - 1 && __syncthreads_and(eq)) {
+        quiet_end();
+        return;
+      }
+      if (!eq && (tid & 31) == 0) a.moving0[tile_id] = a.stamp;
+    }
   }
 
   // ---- phases G1, G2 (learned gate, 2D): features, then the BF16 tensor-core MLP ----
@@ -1205,13 +1319,13 @@ __global__ void __launch_bounds__(TL::NT, 1024 / TL::NT) k_stage(const __grid_co
 // rows are the lower tiles TH of the same CTA size: a CTA of TH costs about
 // 0.6 of one of TL, so the launch's last wave of CTAs ends more evenly across
 // the SMs (the CTAs are scheduled in launch order, the TH rows last).
-template <int NQ_, class TL, class TH>
+template <int GATE, int NQ_, class TL, class TH>
 __global__ void __launch_bounds__(TL::NT, 1024 / TL::NT) k_stage_tail(const __grid_constant__ StageArgs a) {
   static_assert(TL::NT == TH::NT && TL::TX == TH::TX, "one CTA shape");
   if ((int)blockIdx.y < a.rows_full)
-    stage_body<0, NQ_, 0, TL, 0>(a, blockIdx.y, 0);
+    stage_body<GATE, NQ_, 0, TL, 0>(a, blockIdx.y, 0);
   else
-    stage_body<0, NQ_, 0, TH, 1>(a, blockIdx.y - a.rows_full, a.rows_full * TL::TY);
+    stage_body<GATE, NQ_, 0, TH, 1>(a, blockIdx.y - a.rows_full, a.rows_full * TL::TY);
 }
 
 }  // namespace
@@ -1265,7 +1379,7 @@ constexpr int smem_of() {
 
 // the tail-filled 2D launch: room for either tile shape
 constexpr int tail_smem() {
-  return smem_of<0, 6, 0, TileA>() > smem_of<0, 6, 0, TileH>() ? smem_of<0, 6, 0, TileA>() : smem_of<0, 6, 0, TileH>();
+  return smem_of<4, 6, 0, TileA>() > smem_of<4, 6, 0, TileH>() ? smem_of<4, 6, 0, TileA>() : smem_of<4, 6, 0, TileH>();
 }
 
 template <int GATE, int NQ, int MODE, class TL>
@@ -1280,9 +1394,12 @@ cudaError_t fused2d_prepare() {
   cudaError_t e;
   if ((e = allow_smem<0, 6, 0, TileA>()) || (e = allow_smem<1, 6, 0, TileA>()) || (e = allow_smem<2, 6, 0, TileA>()) ||
       (e = allow_smem<3, 6, 0, TileA>()) || (e = allow_smem<0, 6, 0, TileB>()) || (e = allow_smem<3, 6, 0, TileB>()) ||
-      (e = allow_smem<0, 6, 0, TileC>()) || (e = allow_smem<3, 6, 0, TileC>()))
+      (e = allow_smem<0, 6, 0, TileC>()) || (e = allow_smem<3, 6, 0, TileC>()) || (e = allow_smem<4, 6, 0, TileA>()) ||
+      (e = allow_smem<4, 6, 0, TileB>()) || (e = allow_smem<4, 6, 0, TileC>()))
     return e;
-  return cudaFuncSetAttribute(k_stage_tail<6, TileA, TileH>, cudaFuncAttributeMaxDynamicSharedMemorySize, tail_smem());
+  if ((e = cudaFuncSetAttribute(k_stage_tail<0, 6, TileA, TileH>, cudaFuncAttributeMaxDynamicSharedMemorySize, tail_smem())))
+    return e;
+  return cudaFuncSetAttribute(k_stage_tail<4, 6, TileA, TileH>, cudaFuncAttributeMaxDynamicSharedMemorySize, tail_smem());
 }
 
 // Tile rows of a tail-filled 2D launch (tile 3): the number R of TileA rows,
@@ -1427,7 +1544,27 @@ static StageArgs stage_args(const GridDev& g, int stage, double* U, float* U32, 
   a.img_in = 0;
   a.img_out = nullptr;
   a.rows_full = 0;
+  a.moving0 = a.moving1 = nullptr;
+  a.stamp = 0;
   return a;
+}
+
+// Tiles of the finest 2D tiling (and of the tail-filled one).
+int64_t fused2d_max_tiles(const GridDev& g) {
+  return (int64_t)((g.n[0] + TileC::TX - 1) / TileC::TX) * ((g.n[1] + TileC::TY - 1) / TileC::TY + 1);
+}
+
+// Whether a launch looks for quiet tiles: it has several waves of CTAs (with
+// one or two, the slowest tiles are all that counts: 1.2 % lost at 512^2), and
+// the tiles' halos lie in their neighbours, which fails where a periodic axis
+// ends in a tile of less than three cells.
+static bool quiet_tiles(const GridDev& g, int tile, int rows_full) {
+  auto last = [](int n, int t) { return n - (n - 1) / t * t; };
+  const int ty = tile == 1 ? TileB::TY : (tile == 2 ? TileC::TY : TileA::TY);
+  int ly = last(g.n[1], ty);
+  if (tile == 3 && rows_full >= 0 && rows_full * TileA::TY < g.n[1]) ly = last(g.n[1] - rows_full * TileA::TY, TileH::TY);
+  if (fused2d_max_tiles(g) < 8 * 304) return false;
+  return (g.bc[0][0] != WS_BC_PERIODIC || last(g.n[0], TileA::TX) >= NG) && (g.bc[1][0] != WS_BC_PERIODIC || ly >= NG);
 }
 
 // The stage configurations ws_autotune chooses among: tile (0 TileA, 1 TileB,
@@ -1443,10 +1580,15 @@ void launch_stage2d(const GridDev& g, int stage, double* U, float* U32, const fl
                     const GateArgs* gate, const int* run_if, unsigned long long* census, int tile, bool pdl,
                     bool img_in, float* img_out, const CUtensorMap* tmk, const CUtensorMap* tmv,
                     unsigned long long* clear0, unsigned long long* clear1, int rows_full, const CUtensorMap* tmk2,
-                    const CUtensorMap* tmv2, cudaStream_t s) {
+                    const CUtensorMap* tmv2, int* moving, int stamp, cudaStream_t s) {
   StageArgs a = stage_args(g, stage, U, U32, Kin, Kout, dt_fixed, cfl, lmax, dt_out, eps_rel, mood, weights, nbad);
   a.clear0 = clear0;
   a.clear1 = clear1;
+  if (moving && !gate && !census && !run_if && quiet_tiles(g, tile, rows_full)) {
+    a.moving0 = moving;
+    a.moving1 = moving + fused2d_max_tiles(g);
+    a.stamp = stamp;
+  }
   if (tmk && tmv && !gate) {
     a.tma = 1;
     a.tm_k = *tmk;
@@ -1493,8 +1635,16 @@ void launch_stage2d(const GridDev& g, int stage, double* U, float* U32, const fl
       }
     }
     const int hrows = (g.n[1] - rows_full * TileA::TY + TileH::TY - 1) / TileH::TY;
-    launch_kernel(k_stage_tail<6, TileA, TileH>, TileA::NT, tail_smem(), dim3(grid2d<TileA>(g).x, rows_full + hrows),
+    launch_kernel(a.moving0 ? k_stage_tail<4, 6, TileA, TileH> : k_stage_tail<0, 6, TileA, TileH>, TileA::NT, tail_smem(), dim3(grid2d<TileA>(g).x, rows_full + hrows),
                   pdl, s, a);
+    return;
+  }
+  if (a.moving0) {
+    switch (tile) {
+      case 1: launch_k<4, 6, 0, TileB>(grid2d<TileB>(g), pdl, s, a); break;
+      case 2: launch_k<4, 6, 0, TileC>(grid2d<TileC>(g), pdl, s, a); break;
+      default: launch_k<4, 6, 0, TileA>(grid2d<TileA>(g), pdl, s, a); break;
+    }
     return;
   }
   switch (tile) {

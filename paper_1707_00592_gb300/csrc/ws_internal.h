@@ -81,6 +81,8 @@ struct ws_ctx {
   CUtensorMap tmap[10];
   unsigned tmap_ok = 0;
   int tail_rows = 0;            // fused 2D, tile 3: tile rows of the first shape (fused2d_tail_rows)
+  int* moving = nullptr;        // fused 2D: marks of the tiles that are not quiet, stamped with the step's count
+  int stamp = 0;
   bool resident = false;        // fused 2D/3D: carry the FP32 image of U between steps (ws_set_resident)
   float* img[2] = {nullptr, nullptr};  // the two image buffers (one read by a step, one written)
   int img_cur = -1;             // image valid for the next step on img_U, or -1
@@ -207,7 +209,11 @@ void launch_stage2d(const GridDev& g, int stage, double* U, float* U32, const fl
                     const GateArgs* gate, const int* run_if, unsigned long long* census, int tile, bool pdl,
                     bool img_in, float* img_out, const CUtensorMap* tmk, const CUtensorMap* tmv,
                     unsigned long long* clear0, unsigned long long* clear1, int rows_full, const CUtensorMap* tmk2,
-                    const CUtensorMap* tmv2, cudaStream_t s);
+                    const CUtensorMap* tmv2, int* moving, int stamp, cudaStream_t s);
+// moving (nullable): 2 x fused2d_max_tiles(g) marks of the tiles that were not
+// quiet (ws_fused.cu) in the step of a stamp; stamp: this step's, from 1, the
+// same for its three stages and never used before with these marks
+int64_t fused2d_max_tiles(const GridDev& g);
 // rows_full, tmk2, tmv2 (tile 3): the tile rows of the first shape and the
 // descriptors (tile code 4) of the closing rows' boxes
 // clear0, clear1 (nullable): device slots the launch sets to zero once the

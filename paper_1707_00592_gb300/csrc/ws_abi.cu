@@ -140,8 +140,7 @@ void free_all(ws_ctx* c) {
   cudaFree(c->Uhost_dev);
   cudaFree(c->off_dev);
   cudaFree(c->cell_tube);
-  cudaFree(c->chunk_tube);
-  cudaFree(c->chunk_start);
+  cudaFree(c->chunks);
   cudaFree(c->counters);
   cudaFree(c->mood_counts);
   cudaFree(c->mask_off_dev);
@@ -169,26 +168,22 @@ bool tubes(const ws_ctx* c) { return c->grid.ntubes > 0; }
 
 // work items of the persistent mixed-precision tube kernel: chunks of CH cells
 int build_chunks(ws_ctx* c, int config) {
-  int CH = tube_chunk_size(config);
-  std::vector<int64_t> ct;
-  std::vector<int> cs;
+  const int CH = tube_chunk_size(config);
+  std::vector<TubeItem> items;
   for (int64_t t = 0; t < c->td.ntubes; ++t) {
-    int64_t len = c->off_host[t + 1] - c->off_host[t] - 2 * NG;
-    for (int64_t s0 = 0; s0 < len; s0 += CH) {
-      ct.push_back(t);
-      cs.push_back((int)s0);
-    }
+    const int64_t off = c->off_host[t], len = c->off_host[t + 1] - off - 2 * NG;
+    for (int64_t s0 = 0; s0 < len; s0 += CH)
+      items.push_back(TubeItem{off, (int)t, (int)len, (int)s0, (int)items.size(), 0, 0});
   }
-  cudaFree(c->chunk_tube);
-  cudaFree(c->chunk_start);
-  c->chunk_tube = nullptr;
-  c->chunk_start = nullptr;
+  cudaFree(c->chunks);
+  cudaFree(c->counters);
+  c->chunks = nullptr;
+  c->counters = nullptr;
+  const int64_t n = (int64_t)items.size();
   int rc;
-  if ((rc = dalloc(c, &c->chunk_tube, (int64_t)ct.size())) || (rc = dalloc(c, &c->chunk_start, (int64_t)cs.size())))
-    return rc;
-  CK(c, cudaMemcpy(c->chunk_tube, ct.data(), ct.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
-  CK(c, cudaMemcpy(c->chunk_start, cs.data(), cs.size() * sizeof(int), cudaMemcpyHostToDevice));
-  c->nchunks = (int64_t)ct.size();
+  if ((rc = dalloc(c, &c->chunks, 3 * n)) || (rc = dalloc(c, &c->counters, 8 + 2 * n))) return rc;
+  CK(c, cudaMemcpy(c->chunks, items.data(), n * sizeof(TubeItem), cudaMemcpyHostToDevice));
+  c->nchunks = n;
   c->tube_config = config;
   return WS_OK;
 }
@@ -355,15 +350,13 @@ int step_device(ws_ctx* c, double* U, double dt) {
   if (tubes(c) && mixed(c)) {
     const int64_t nt = c->td.ntubes;
     CK(c, cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long) * nt, c->stream));
-    CK(c, cudaMemsetAsync(c->counters, 0, 3 * sizeof(unsigned), c->stream));
+    CK(c, cudaMemsetAsync(c->counters, 0, (8 + 2 * c->nchunks) * sizeof(unsigned), c->stream));
+    const TubeWork w{c->chunks, c->nchunks, c->counters, (int*)(c->counters + 8), c->chunks + c->nchunks};
     for (int s = 0; s < 3; ++s) {
       KScope k(c, WS_K_FACE);
-      const float* Kin = s == 1 ? c->Ka : c->Kb;
-      float* Kout = s == 0 ? c->Ka : c->Kb;
-      launch_tubes_stage_mixed(c->td, c->tube_config, s, U, c->Q32, Kin, Kout, dt, c->opts.cfl, c->lmax, c->dt_dev,
-                               c->chunk_tube, c->chunk_start, c->nchunks, c->counters + s,
-                               c->mask + (int64_t)s * c->nmask, (float)c->opts.eps, c->opts.mood, c->opts.weights,
-                               c->nbad, c->stream);
+      launch_tubes_stage_mixed(c->td, c->tube_config, s, U, c->Q32, c->Ka, c->Kb, dt, c->opts.cfl, c->lmax, c->dt_dev,
+                               w, c->mask, c->nmask, (float)c->opts.eps, c->opts.mood, c->opts.weights, c->nbad,
+                               c->stream);
     }
     c->last_stages = 3;
     return check_launch(c, "mixed tube stage");
@@ -627,7 +620,7 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
     c->off_host = off;
     if (op.precision == WS_PREC_MIXED) {
       if ((rc = dalloc(c, &c->Q32, 5 * total)) || (rc = dalloc(c, &c->Ka, 5 * total)) ||
-          (rc = dalloc(c, &c->Kb, 5 * total)) || (rc = dalloc(c, &c->counters, 3)) || (rc = build_chunks(c, 2)))
+          (rc = dalloc(c, &c->Kb, 5 * total)) || (rc = build_chunks(c, 2)))
         goto bad;
     }
   }

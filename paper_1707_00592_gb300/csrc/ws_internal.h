@@ -44,6 +44,21 @@ struct TubesDev {
   const int* cell_tube; // device, tube index of every padded cell
 };
 
+// A chunk of a tube: work item of the mixed-precision tube stages.
+struct alignas(16) TubeItem {
+  int64_t off;          // the tube's first padded cell
+  int tube, len;        // its index and interior cells
+  int c0, index;        // first cell of the chunk (tube-local), place among all items (chunks of a tube in order)
+  int pad0, pad1;
+};
+struct TubeWork {
+  const TubeItem* items;
+  int64_t nitems;
+  unsigned* counters;   // zeroed before a step: work counters of the stages [0..2], items listed for stages 1 and 2 [3, 4]
+  int* listed;          // zeroed before a step: whether an item is listed, for stage 1, then stage 2
+  TubeItem* list;       // the items listed for stage 1, then (at nitems) for stage 2
+};
+
 }  // namespace ws
 
 struct ws_ctx {
@@ -106,10 +121,9 @@ struct ws_ctx {
   int* cell_tube = nullptr;
   std::vector<int64_t> off_host;   // tube offsets
   int tube_config = 2;             // mixed tubes: autotuned (chunk, threads) configuration
-  int64_t* chunk_tube = nullptr;   // device: work item -> tube
-  int* chunk_start = nullptr;      // device: work item -> first cell of the chunk
+  ws::TubeItem* chunks = nullptr;  // device: the work items, then the lists of stages 1 and 2
   int64_t nchunks = 0;
-  unsigned* counters = nullptr;    // device: 3 work counters (one per stage)
+  unsigned* counters = nullptr;    // device: 8 counters, then 2 x nchunks marks (TubeWork)
   // measurement: event pairs around launches, launch counts per kernel class
   bool prof_on = false;
   std::vector<cudaEvent_t> ev;  // 2 per recorded launch
@@ -250,11 +264,11 @@ void launch_restore(const int* redo, const double* src, double* dst, int64_t n, 
 // ---- batched tubes, mixed precision, persistent (ws_tubes_mixed.cu) ----
 extern const int kNumTubeConfigs;
 int tube_chunk_size(int config);
-void launch_tubes_stage_mixed(const TubesDev& t, int config, int stage, double* U, float* U32, const float* Kin,
-                              float* Kout, double dt_fixed, double cfl, unsigned long long* lmax, double* dt_out,
-                              const int64_t* chunk_tube, const int* chunk_start, int64_t nitems, unsigned* counter,
-                              uint8_t* mask, float eps_rel, int mood, int weights, unsigned long long* nbad,
-                              cudaStream_t s);
+// mask: the first of the three stages' records, nmask bytes each
+void launch_tubes_stage_mixed(const TubesDev& t, int config, int stage, double* U, float* U32, float* Ka, float* Kb,
+                              double dt_fixed, double cfl, unsigned long long* lmax, double* dt_out,
+                              const TubeWork& work, uint8_t* mask, int64_t nmask, float eps_rel, int mood, int weights,
+                              unsigned long long* nbad, cudaStream_t s);
 
 // ---- learned gate (ws_learned.cu) ----
 void launch_face_samples(const GridDev& g, int d, const float* Q, int64_t stride, int64_t out0, int64_t max_out,

@@ -134,14 +134,16 @@ void free_all(ws_ctx* c) {
   }
   cudaFree(c->mask);
   cudaFree(c->dt_dev);
-  cudaFree(c->lmax);
-  cudaFree(c->nbad);
+  if (!c->zeroed) {
+    cudaFree(c->lmax);
+    cudaFree(c->nbad);
+  }
+  cudaFree(c->zeroed);
   cudaFree(c->census);
   cudaFree(c->Uhost_dev);
   cudaFree(c->off_dev);
   cudaFree(c->cell_tube);
   cudaFree(c->chunks);
-  cudaFree(c->counters);
   cudaFree(c->mood_counts);
   cudaFree(c->mask_off_dev);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
@@ -176,12 +178,27 @@ int build_chunks(ws_ctx* c, int config) {
       items.push_back(TubeItem{off, (int)t, (int)len, (int)s0, (int)items.size(), 0, 0});
   }
   cudaFree(c->chunks);
-  cudaFree(c->counters);
   c->chunks = nullptr;
-  c->counters = nullptr;
-  const int64_t n = (int64_t)items.size();
+  const int64_t n = (int64_t)items.size(), nt = c->td.ntubes;
   int rc;
-  if ((rc = dalloc(c, &c->chunks, 3 * n)) || (rc = dalloc(c, &c->counters, 8 + 2 * n))) return rc;
+  if ((rc = dalloc(c, &c->chunks, 3 * n))) return rc;
+  // nbad, lmax and the counters lie in one block; the first call brings the
+  // first two over from their own
+  unsigned long long* z = nullptr;
+  if ((rc = dalloc(c, &z, 1 + nt + 4 + n))) return rc;
+  if (c->zeroed) {
+    cudaFree(c->zeroed);
+  } else {
+    cudaFree(c->nbad);
+    cudaFree(c->lmax);
+  }
+  c->zeroed = z;
+  c->zeroed_bytes = (1 + nt + 4 + n) * (int64_t)sizeof(unsigned long long);
+  c->nbad = z;
+  c->lmax = z + 1;
+  c->counters = reinterpret_cast<unsigned*>(z + 1 + nt);
+  c->nbad_last = nullptr;
+  CK(c, cudaMemset(z, 0, c->zeroed_bytes));
   CK(c, cudaMemcpy(c->chunks, items.data(), n * sizeof(TubeItem), cudaMemcpyHostToDevice));
   c->nchunks = n;
   c->tube_config = config;
@@ -346,11 +363,10 @@ int step_device(ws_ctx* c, double* U, double dt) {
   int rc;
   c->nbad_last = c->nbad;
   // a plain fused step clears (or rotates) its own counter, an FP64 grid step its own
-  if (!(c->fused && !c->learned_on) && (mixed(c) || tubes(c))) CK(c, cudaMemsetAsync(c->nbad, 0, sizeof(unsigned long long), c->stream));
+  // and mixed tubes with their other counters
+  if (!(c->fused && !c->learned_on) && mixed(c) != tubes(c)) CK(c, cudaMemsetAsync(c->nbad, 0, sizeof(unsigned long long), c->stream));
   if (tubes(c) && mixed(c)) {
-    const int64_t nt = c->td.ntubes;
-    CK(c, cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long) * nt, c->stream));
-    CK(c, cudaMemsetAsync(c->counters, 0, (8 + 2 * c->nchunks) * sizeof(unsigned), c->stream));
+    CK(c, cudaMemsetAsync(c->zeroed, 0, c->zeroed_bytes, c->stream));
     const TubeWork w{c->chunks, c->nchunks, c->counters, (int*)(c->counters + 8), c->chunks + c->nchunks};
     for (int s = 0; s < 3; ++s) {
       KScope k(c, WS_K_FACE);
@@ -620,7 +636,7 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
     c->off_host = off;
     if (op.precision == WS_PREC_MIXED) {
       if ((rc = dalloc(c, &c->Q32, 5 * total)) || (rc = dalloc(c, &c->Ka, 5 * total)) ||
-          (rc = dalloc(c, &c->Kb, 5 * total)) || (rc = build_chunks(c, 2)))
+          (rc = dalloc(c, &c->Kb, 5 * total)) || (rc = build_chunks(c, tube_default_config(total))))
         goto bad;
     }
   }

@@ -124,6 +124,8 @@ struct ws_ctx {
   ws::TubeItem* chunks = nullptr;  // device: the work items, then the lists of stages 1 and 2
   int64_t nchunks = 0;
   unsigned* counters = nullptr;    // device: 8 counters, then 2 x nchunks marks (TubeWork)
+  unsigned long long* zeroed = nullptr;  // mixed tubes: what a step zeroes in one go -- nbad, lmax, counters (all in here)
+  int64_t zeroed_bytes = 0;
   // measurement: event pairs around launches, launch counts per kernel class
   bool prof_on = false;
   std::vector<cudaEvent_t> ev;  // 2 per recorded launch
@@ -264,6 +266,7 @@ void launch_restore(const int* redo, const double* src, double* dst, int64_t n, 
 // ---- batched tubes, mixed precision, persistent (ws_tubes_mixed.cu) ----
 extern const int kNumTubeConfigs;
 int tube_chunk_size(int config);
+int tube_default_config(int64_t cells);
 // mask: the first of the three stages' records, nmask bytes each
 void launch_tubes_stage_mixed(const TubesDev& t, int config, int stage, double* U, float* U32, float* Ka, float* Kb,
                               double dt_fixed, double cfl, unsigned long long* lmax, double* dt_out,

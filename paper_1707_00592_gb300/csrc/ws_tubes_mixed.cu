@@ -24,7 +24,7 @@
 // While a CTA works on an item, its first thread fetches the next one's
 // description and CFL rate step by step with asynchronous copies, so that no
 // item starts with a chain of dependent loads.  4096 tubes (9.4 M cells, half
-// of them quiet): 1034 -> TUBE_NOW us per step.
+// of them quiet): 1034 -> 607 us per step.
 #include <cuda_runtime.h>
 
 #include "face_fp32.cuh"
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) k_tube_stage(const __grid_con
   };
   unsigned nxt = 0;
   if (tid == 0) {
-    nxt = atomicAdd(counter, 1u);
+    nxt = blockIdx.x;  // the first item is the CTA's own, the counter hands out those after the first wave
     fetch_item(nxt);
     fetch_rate(nxt);
     take(nxt);
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) k_tube_stage(const __grid_con
   for (;;) {
     __syncthreads();
     if (!S.more) break;
-    if (tid == 0) nxt = atomicAdd(counter, 1u);
+    if (tid == 0) nxt = gridDim.x + atomicAdd(counter, 1u);
     const int64_t tube = S.now.tube;
     const int64_t off = S.now.off;
     const int len = S.now.len;
@@ -345,10 +345,15 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) k_tube_stage(const __grid_con
         for (int m = 0; m < NQ; ++m) a.Kout[m * N + gi] = a.Kin[m * N + gi] + inc[m];
       } else {
         float d[NQ];
+        bool moves = false;
 #pragma unroll
         for (int m = 0; m < NQ; ++m) {
           d[m] = dt * fmaf(1.0f / 6.0f, a.Kin[m * N + gi], (2.0f / 3.0f) * inc[m]);
-          a.U[m * N + gi] = a.U[m * N + gi] + f32_to_f64(d[m]);
+          moves = moves || d[m] != 0.0f;
+        }
+        if (moves) {  // (a cell of the chunks beside the waves often does not)
+#pragma unroll
+          for (int m = 0; m < NQ; ++m) a.U[m * N + gi] = a.U[m * N + gi] + f32_to_f64(d[m]);
         }
         const float* V = a.U32;
         float rho = V[gi] + d[0], mu = V[N + gi] + d[1];
@@ -387,6 +392,14 @@ const int kTubeConfigs[][2] = {{255, 128}, {255, 256}, {511, 256}, {511, 512}, {
 const int kNumTubeConfigs = 5;
 
 int tube_chunk_size(int config) { return kTubeConfigs[config][0]; }
+
+// The configuration of a new context, for `cells` cells: the smallest chunks
+// leave the most cells out where the tubes are quiet (4096 tubes, half of their
+// cells quiet: 607 us per step, against 643, 674, 839 and 864 us for the
+// others in turn; none quiet: 1378 against 1363 and 1344).  A batch that does
+// not fill the GPU with them takes a face to a thread (32 tubes of 100 to 1000
+// cells: 29 us against 36).
+int tube_default_config(int64_t cells) { return cells >= 255LL * 152 * 8 ? 0 : 1; }
 
 void launch_tubes_stage_mixed(const TubesDev& t, int config, int stage, double* U, float* U32, float* Ka, float* Kb,
                               double dt_fixed, double cfl, unsigned long long* lmax, double* dt_out,

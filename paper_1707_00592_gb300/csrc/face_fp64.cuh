@@ -65,11 +65,11 @@ __device__ __forceinline__ double mul(double a, double b, uint32_t& rg) {
 }
 template <int PI>
 __device__ __forceinline__ double sqroot(double x, uint32_t& rg) {
-  return PI == NATIVE ? sqrt(x) : isqrt(x, rg);
+  return PI == NATIVE ? sqrt(x) : (PI == CHAIN ? root_call(x) : isqrt(x, rg));
 }
 template <int PI>
 __device__ __forceinline__ double quot(double a, double b, uint32_t& rg) {
-  return PI == NATIVE ? a / b : idiv(a, b, rg);
+  return PI == NATIVE ? a / b : (PI == CHAIN ? divide_call(a, b) : idiv(a, b, rg));
 }
 // A launch of many CTAs (NQ chunks of faces each) is bound by the pipes, and
 // its products go to the integer pipe; one of few CTAs is bound by the length
@@ -272,8 +272,10 @@ __device__ __forceinline__ bool admissible(const double* q) {
 // Where the six cells of a lane pair's face lie: cell i-2+j at base + j st of
 // every primitive field; field m of the sweep frame (rho, u_n, u_t.., p,
 // Gamma, Pi) starts at q + fld(m) N, the sound speed at q + NQ N.
-template <int NQ>
+// SH: the fields lie in shared memory.
+template <int NQ_, bool SH_ = false>
 struct Faces {
+  static constexpr int NQ = NQ_;
   const double* q;
   int64_t N, base, st;
   int d;
@@ -282,12 +284,15 @@ struct Faces {
     if (m == 1) return 1 + d;
     return m - 2 < d ? m - 1 : m;  // tangential velocities in increasing axis order
   }
-  __device__ __forceinline__ double at(int f, int j) const { return __ldg(q + (int64_t)f * N + base + j * st); }
+  __device__ __forceinline__ double at(int f, int j) const {
+    const double* p = q + (int64_t)f * N + base + j * st;
+    return SH_ ? *p : __ldg(p);
+  }
 };
 
 // The MOOD retry of one side: 3rd order, then the cell's own state.  Rare.
-template <int NQ>
-__device__ __noinline__ int retry(const Faces<NQ> fc, int side, double eps, int weights, double* q) {
+template <int NQ, bool SH>
+__device__ __noinline__ int retry(const Faces<NQ, SH> fc, int side, double eps, int weights, double* q) {
   double qc[6][NQ];
 #pragma unroll 1
   for (int j = 0; j < 6; ++j)
@@ -437,8 +442,8 @@ struct FaceSmem {
 };
 
 // The reconstruction of characteristic variable r on a warp's lane pairs.
-template <int NQ, Scheme SC, int PI>
-__device__ __forceinline__ double reconstruct(const Faces<NQ>& fc, int r, double eps, int weights) {
+template <int NQ, Scheme SC, int PI, bool SH>
+__device__ __forceinline__ double reconstruct(const Faces<NQ, SH>& fc, int r, double eps, int weights) {
   constexpr int IP = NQ - 3;
   const int side = threadIdx.x & 1;
   auto cell = [&](int k) { return side ? 5 - k : k; };  // this side's stencil cell k
@@ -447,7 +452,7 @@ __device__ __forceinline__ double reconstruct(const Faces<NQ>& fc, int r, double
     const int s1 = fc.fld(1);
     const double c = fc.at(NQ, cell(2)), s2 = c + partner(c);  // 2 c_bar
     if (r == 1) {
-      const double L1p = divide(-4.0, __dmul_rn(s2, s2));  // -1/c_bar^2
+      const double L1p = PI == CHAIN ? divide_call(-4.0, __dmul_rn(s2, s2)) : divide(-4.0, __dmul_rn(s2, s2));  // -1/c_bar^2
 #pragma unroll
       for (int k = 0; k < 3; ++k) v[k] = fc.at(0, cell(k)) + __dmul_rn(L1p, fc.at(IP, cell(k)));
     } else {
@@ -477,20 +482,22 @@ __device__ __forceinline__ double reconstruct(const Faces<NQ>& fc, int r, double
 
 // The Riemann problem of a warp's lane pairs from the reconstructed
 // characteristics w; code: this side's MOOD level.
-template <int NQ, int PI>
-__device__ __forceinline__ void solve(const Faces<NQ>& fc, const double (&w)[NQ], double eps, int mood, int weights,
+template <int NQ, int PI, bool SH>
+__device__ __forceinline__ void solve(const Faces<NQ, SH>& fc, const double (&w)[NQ], double eps, int mood, int weights,
                                       double (&out)[(NQ + 2) / 2], int& code) {
   const int side = threadIdx.x & 1, own = 2 + side;
   double q[NQ];
   {
     const double c = fc.at(NQ, own), s2 = c + partner(c);
     const double rho = fc.at(0, own), s1 = rho + partner(rho);
-    back_project<NQ>(w, divide(4.0, __dmul_rn(s2, s2)), divide(4.0, __dmul_rn(s1, s2)), q);
+    const double cc = __dmul_rn(s2, s2), rc = __dmul_rn(s1, s2);
+    back_project<NQ>(w, PI == CHAIN ? divide_call(4.0, cc) : divide(4.0, cc),
+                     PI == CHAIN ? divide_call(4.0, rc) : divide(4.0, rc), q);
   }
   code = 0;
   if (mood && !admissible<NQ>(q)) {
     double q3[NQ];
-    code = retry<NQ>(fc, side, eps, weights, q3);
+    code = retry(fc, side, eps, weights, q3);
 #pragma unroll
     for (int m = 0; m < NQ; ++m) q[m] = q3[m];
   }
@@ -516,7 +523,7 @@ __device__ __forceinline__ void cta_faces(FaceSmem<NQ, CH>& sm, double eps, int 
   int code;
 #pragma unroll
   for (int m = 0; m < NQ; ++m) w[m] = sm.w[k][m][lane];
-  const Faces<NQ> fc = at(k);
+  const auto fc = at(k);
   solve<NQ, PI>(fc, w, eps, mood, weights, out, code);
   done(k, fc, out, code);
 }

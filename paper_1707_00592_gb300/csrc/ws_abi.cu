@@ -362,9 +362,9 @@ int step_device(ws_ctx* c, double* U, double dt) {
   const GridDev& g = c->gd;
   int rc;
   c->nbad_last = c->nbad;
-  // a plain fused step clears (or rotates) its own counter, an FP64 grid step its own
-  // and mixed tubes with their other counters
-  if (!(c->fused && !c->learned_on) && mixed(c) != tubes(c)) CK(c, cudaMemsetAsync(c->nbad, 0, sizeof(unsigned long long), c->stream));
+  // FP64 tubes, a gated step and the general mixed path (the others clear their own counter)
+  if (mixed(c) ? !tubes(c) && (!c->fused || c->learned_on) && g.ndim > 1 : tubes(c))
+    CK(c, cudaMemsetAsync(c->nbad, 0, sizeof(unsigned long long), c->stream));
   if (tubes(c) && mixed(c)) {
     CK(c, cudaMemsetAsync(c->zeroed, 0, c->zeroed_bytes, c->stream));
     const TubeWork w{c->chunks, c->nchunks, c->counters, (int*)(c->counters + 8), c->chunks + c->nchunks};
@@ -414,6 +414,20 @@ int step_device(ws_ctx* c, double* U, double dt) {
     }
     c->last_stages = 3;
     return WS_OK;
+  }
+  if (g.ndim == 1) {  // a launch per stage
+    for (int s = 0; s < 3; ++s) {
+      KScope k(c, WS_K_FACE);
+      uint8_t* mb = c->mask + (int64_t)s * c->nmask;
+      if (mixed(c))
+        launch_line_mixed(g, s, U, c->Fh32[0], c->S1, mb, (float)c->opts.eps, c->opts.mood, c->opts.weights, dt,
+                          c->opts.cfl, c->lmax, c->dt_dev, c->nbad, c->stream);
+      else
+        launch_line_fp64(g, s, U, c->Fh[0], c->S1, mb, c->opts.eps, c->opts.mood, c->opts.weights, dt, c->opts.cfl,
+                         c->lmax, c->dt_dev, c->nbad, c->stream);
+    }
+    c->last_stages = 3;
+    return check_launch(c, "1D stage");
   }
   if (!mixed(c)) {
     // three launches per stage.  Stage 0's first zeroes the inadmissible-cell

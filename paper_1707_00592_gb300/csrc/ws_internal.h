@@ -179,7 +179,18 @@ void launch_mood_count(const uint8_t* mask, int64_t n, int64_t nstage, const int
 void launch_face_fp64(const GridDev& g, const double* Q, double* const Fh[3], double* const us[3],
                       uint8_t* const mask[3], double eps, int mood, int weights, cudaStream_t s);
 
+// one RK stage of a 1D grid.  L: nv fields of n values (stage 0 writes them),
+// U2: like U (stage 1 writes it); lmax is zero before stage 0 and after stage 2,
+// dt receives the step in stage 1, stage 0 zeroes nbad
+void launch_line_fp64(const GridDev& g, int stage, double* U, double* L, double* U2, uint8_t* mask, double eps, int mood,
+                      int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt,
+                      unsigned long long* nbad, cudaStream_t s);
+
 // ---- mixed-precision sweep (ws_mixed.cu, FMA allowed) ----
+// the same in mixed precision
+void launch_line_mixed(const GridDev& g, int stage, double* U, float* L, double* U2, uint8_t* mask, float eps_rel, int mood,
+                       int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt,
+                       unsigned long long* nbad, cudaStream_t s);
 void launch_prim32(const GridDev& g, const double* U, float* Q, cudaStream_t s);
 void launch_cfl32(const GridDev& g, const float* Q, unsigned long long* lmax, cudaStream_t s);
 void launch_face_mixed(const GridDev& g, int d, const float* Q, float* Fh, float* us, uint8_t* mask, float eps_rel,

@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include "face_fp32.cuh"
+#include "fp64_pipes.cuh"
 #include "ws_internal.h"
 
 namespace ws {
@@ -199,6 +200,135 @@ __global__ void k_update_mixed(GridDev g, int stage, const double* Un, const dou
   }
 }
 
+// One RK stage of a 1D grid in one launch: primitives, faces and update of
+// LF faces and the LF - 1 cells between them (neighbouring CTAs share a face),
+// with the arithmetic of the general kernels above.  Boundary conditions are
+// applied on load.  Stage 0 leaves L(U) and the CFL rate, stage 1 forms
+// U1 = U + dt L from them on load and leaves U2, stage 2 updates U.  Three
+// launches per step instead of the 14 and two memsets of the general path.
+constexpr int LF = 128;
+
+struct LineArgs {
+  int n, stage;
+  int64_t N;                 // padded cells of a field
+  int bc[2];
+  double dx, cfl, dt_fixed;
+  WenoParams P;
+  int mood;
+  double* U;
+  float* L;                  // n values per field
+  double* U2;                // laid out like U
+  uint8_t* mask;             // nullable
+  unsigned long long* lmax;  // zero before stage 0; stage 2 leaves it zero
+  double* dt;
+  unsigned long long* nbad;  // stage 0 sets it to zero
+};
+
+__global__ void __launch_bounds__(LF) k_line32(const __grid_constant__ LineArgs a) {
+  constexpr int C = LF + 5;
+  __shared__ float prim[6][C], flux[6][LF];  // cell c of the CTA is cell f0 - 3 + c
+  __shared__ double cons[5][C];
+  __shared__ double dt_sh;
+  __shared__ float red[LF / 32];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int tid = threadIdx.x, n = a.n;
+  const int f0 = blockIdx.x * (LF - 1);
+  if (tid == 0) {
+    if (a.stage == 1) {
+      dt_sh = a.dt_fixed > 0.0 ? a.dt_fixed : fp64::divide(a.cfl, __longlong_as_double((long long)*a.lmax));
+      if (blockIdx.x == 0) *a.dt = dt_sh;
+    } else if (a.stage == 2) {
+      dt_sh = *a.dt;
+      if (blockIdx.x == 0) *a.lmax = 0ULL;
+    } else if (blockIdx.x == 0) {
+      *a.nbad = 0ULL;
+    }
+  }
+  if (a.stage != 0) __syncthreads();
+  const float idx = (float)(1.0 / a.dx), dt = a.stage != 0 ? (float)dt_sh : 0.0f;
+  float best = 0.0f;
+  for (int c = tid; c < C && f0 - 3 + c < n + NG; c += LF) {
+    const int x = f0 - 3 + c;
+    int m = x;
+    bool flip = false;
+    if (x < 0 || x >= n) {
+      const int kind = a.bc[x < 0 ? 0 : 1];
+      m = x < 0 ? 0 : n - 1;
+      if (kind == WS_BC_PERIODIC) m = x < 0 ? x + n : x - n;
+      if (kind == WS_BC_REFLECTIVE) {
+        m = x < 0 ? -1 - x : 2 * n - 1 - x;
+        flip = true;
+      }
+    }
+    double u[5];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+      u[f] = (a.stage == 2 ? a.U2 : a.U)[f * a.N + NG + m];
+      if (a.stage == 1) u[f] = rk_stage(0, u[f], u[f], dt * a.L[(int64_t)f * n + m]);
+      if (flip && f == 1) u[f] = -u[f];
+      cons[f][c] = u[f];
+    }
+    float q[5], cs;
+    cons_to_prim32<1>(u, q, cs);
+#pragma unroll
+    for (int f = 0; f < 5; ++f) prim[f][c] = q[f];
+    prim[5][c] = cs;
+    if (a.stage == 0 && x >= 0 && x < n) {
+      const float lam = fmaf(fabsf(q[1]) + cs, idx, 0.0f);
+      if (!(lam <= best)) best = lam;  // NaN propagates
+    }
+  }
+  if (a.stage == 0 && a.dt_fixed <= 0.0) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float v = __shfl_xor_sync(0xffffffffu, best, o);
+      if (!(v <= best)) best = v;
+    }
+    if ((tid & 31) == 0) red[tid >> 5] = best;
+  }
+  __syncthreads();
+  if (a.stage == 0 && a.dt_fixed <= 0.0 && tid == 0) {
+    for (int w = 1; w < LF / 32; ++w)
+      if (!(red[w] <= best)) best = red[w];
+    atomicMax(a.lmax, (unsigned long long)__double_as_longlong((double)best));
+  }
+  if (f0 + tid <= n) {
+    float qc[6][5], cc[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+#pragma unroll
+      for (int m = 0; m < 5; ++m) qc[j][m] = prim[m][tid + j];
+      cc[j] = prim[5][tid + j];
+    }
+    float Fhat[5], ustar;
+    int cl, cr;
+    face<5>(qc, cc, a.P, a.mood, Fhat, ustar, cl, cr);
+#pragma unroll
+    for (int m = 0; m < 5; ++m) flux[m][tid] = Fhat[m];
+    flux[5][tid] = ustar;
+    if (a.mask) a.mask[f0 + tid] = (uint8_t)(cl | (cr << 2));
+  }
+  __syncthreads();
+  if (tid == LF - 1 || f0 + tid >= n) return;
+  const int64_t x = f0 + tid;
+  const float du = (flux[5][tid + 1] - flux[5][tid]) * idx;
+  double out[5];
+#pragma unroll
+  for (int f = 0; f < 5; ++f) {
+    float L = fmaf(-(flux[f][tid + 1] - flux[f][tid]), idx, 0.0f);
+    if (f >= 3) L = fmaf(prim[f][tid + 3], 0.0f + du, L);
+    if (a.stage == 0)
+      a.L[f * n + x] = L;
+    else
+      out[f] = rk_stage(a.stage, a.U[f * a.N + NG + x], cons[f][tid + 3], dt * L);
+  }
+  if (a.stage == 0) return;
+#pragma unroll
+  for (int f = 0; f < 5; ++f) (a.stage == 1 ? a.U2 : a.U)[f * a.N + NG + x] = out[f];
+  if (a.stage == 2 && !admissible_cons<1>(out)) atomicAdd(a.nbad, 1ULL);
+}
+
 // max over interior cells of sum_d (|u_d| + c)/dx_d from the FP32 cache
 template <int NDIM>
 __global__ void k_cfl32(GridDev g, const float* __restrict__ Q, unsigned long long* lmax) {
@@ -345,6 +475,23 @@ void launch_update_mixed(const GridDev& g, int stage, const double* Un, const do
                                          nbad);
       break;
   }
+}
+
+void launch_line_mixed(const GridDev& g, int stage, double* U, float* L, double* U2, uint8_t* mask, float eps_rel, int mood,
+                       int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt,
+                       unsigned long long* nbad, cudaStream_t s) {
+  const LineArgs a{g.n[0], stage, g.N, {g.bc[0][0], g.bc[0][1]}, g.dx[0], cfl, dt_fixed, weno_params(eps_rel, weights),
+                   mood, U, L, U2, mask, lmax, dt, nbad};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((a.n + LF - 2) / (LF - 1)));
+  cfg.blockDim = dim3(LF);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_line32, a);
 }
 
 }  // namespace ws

@@ -8,6 +8,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -87,6 +88,49 @@ int dalloc(ws_ctx* c, T** p, int64_t count) {
   return WS_OK;
 }
 
+// Mapped host memory for the steps of the process's grid contexts: a page of
+// 64 slots, a cache line each, allocated once (which takes longer than the rest
+// of a small context).  A context without a slot has its step copied.
+class DtSlots {
+ public:
+  void take(double** host, double** dev) {
+    std::lock_guard<std::mutex> lock(m_);
+    *host = *dev = nullptr;
+    if (!page_ && !tried_) {
+      tried_ = true;
+      if (cudaHostAlloc((void**)&page_, kSlots * kStride * sizeof(double), cudaHostAllocMapped | cudaHostAllocPortable) !=
+          cudaSuccess) {
+        cudaGetLastError();
+        page_ = nullptr;
+      }
+    }
+    for (int k = 0; page_ && k < kSlots; ++k) {
+      if (used_ >> k & 1u) continue;
+      double* h = page_ + k * kStride;
+      if (cudaHostGetDevicePointer((void**)dev, h, 0) != cudaSuccess) {
+        cudaGetLastError();
+        *dev = nullptr;
+        return;
+      }
+      used_ |= 1ULL << k;
+      *host = h;
+      return;
+    }
+  }
+  void give(double* host) {
+    std::lock_guard<std::mutex> lock(m_);
+    if (host) used_ &= ~(1ULL << ((host - page_) / kStride));
+  }
+
+ private:
+  static constexpr int kSlots = 64, kStride = 8;
+  std::mutex m_;
+  double* page_ = nullptr;
+  bool tried_ = false;
+  unsigned long long used_ = 0;
+};
+DtSlots dt_slots;
+
 // Records an event pair around the launches of its scope and counts the kernel
 // launches of its class, while profiling is on.
 struct KScope {
@@ -134,6 +178,7 @@ void free_all(ws_ctx* c) {
   }
   cudaFree(c->mask);
   cudaFree(c->dt_dev);
+  dt_slots.give(c->dt_host);
   if (!c->zeroed) {
     cudaFree(c->lmax);
     cudaFree(c->nbad);
@@ -249,7 +294,8 @@ int update(ws_ctx* c, int stage, const double* Un, const double* Us, double* Uou
   if (mixed(c))
     launch_update_mixed(c->gd, stage, Un, Us, Uout, c->Fh32, c->us32, c->Q32, c->dt_dev, c->nbad, c->stream);
   else
-    launch_update(c->gd, stage, Un, Us, Uout, c->Fh, c->us, dt, c->opts.cfl, c->lmax, c->dt_dev, c->nbad, c->stream);
+    launch_update(c->gd, stage, Un, Us, Uout, c->Fh, c->us, dt, c->opts.cfl, c->lmax, c->dt_dev,
+                  c->dt_host_dev, c->nbad, c->stream);
   return check_launch(c, "update");
 }
 
@@ -339,7 +385,7 @@ int fused_run3(ws_ctx* c, double* U, double dt, const GateArgs* gate, const int*
                      mb + c->mask_off[1], mb + c->mask_off[2], (float)c->opts.eps, c->opts.mood, c->opts.weights, nbad,
                      census, c->stage_tile, c->stage_sched == 0, s == 0 && img_in, s == 2 ? img_out : nullptr,
                      s == 2 ? clr0 : nullptr, s == 2 ? clr1 : nullptr, tmk, tmv, map2_of(c, tmk), map2_of(c, tmv),
-                     c->stream);
+                     one_scope ? c->dt_host_dev : nullptr, c->stream);
     } else {
       const CUtensorMap *tmk = map_of(c, Kin), *tmv = map_of(c, u32);
       if (!tmk || !tmv) tmk = tmv = nullptr;
@@ -347,7 +393,7 @@ int fused_run3(ws_ctx* c, double* U, double dt, const GateArgs* gate, const int*
                      mb + c->mask_off[1], (float)c->opts.eps, c->opts.mood, c->opts.weights, nbad, gate, run_if,
                      census, c->stage_tile, c->stage_sched == 0, s == 0 && img_in, s == 2 ? img_out : nullptr, tmk,
                      tmv, s == 2 ? clr0 : nullptr, s == 2 ? clr1 : nullptr, c->tail_rows, map2_of(c, tmk),
-                     map2_of(c, tmv), moving, c->stamp, c->stream);
+                     map2_of(c, tmv), moving, c->stamp, one_scope ? c->dt_host_dev : nullptr, c->stream);
     }
   }
   return check_launch(c, "fused stage");
@@ -362,6 +408,7 @@ int step_device(ws_ctx* c, double* U, double dt) {
   const GridDev& g = c->gd;
   int rc;
   c->nbad_last = c->nbad;
+  c->dt_mapped = false;
   // FP64 tubes, a gated step and the general mixed path (the others clear their own counter)
   if (mixed(c) ? !tubes(c) && (!c->fused || c->learned_on) && g.ndim > 1 : tubes(c))
     CK(c, cudaMemsetAsync(c->nbad, 0, sizeof(unsigned long long), c->stream));
@@ -397,6 +444,7 @@ int step_device(ws_ctx* c, double* U, double dt) {
   if (c->fused) {
     if (!c->learned_on) {
       if ((rc = fused_run3(c, U, dt, nullptr, nullptr))) return rc;
+      c->dt_mapped = c->dt_host != nullptr;
     } else {
       // gated step, then on the device: keep or redo it without the gate
       // (restored from the backup taken in stage 0), with no host round trip
@@ -421,11 +469,12 @@ int step_device(ws_ctx* c, double* U, double dt) {
       uint8_t* mb = c->mask + (int64_t)s * c->nmask;
       if (mixed(c))
         launch_line_mixed(g, s, U, c->Fh32[0], c->S1, mb, (float)c->opts.eps, c->opts.mood, c->opts.weights, dt,
-                          c->opts.cfl, c->lmax, c->dt_dev, c->nbad, c->stream);
+                          c->opts.cfl, c->lmax, c->dt_dev, c->dt_host_dev, c->nbad, c->stream);
       else
         launch_line_fp64(g, s, U, c->Fh[0], c->S1, mb, c->opts.eps, c->opts.mood, c->opts.weights, dt, c->opts.cfl,
-                         c->lmax, c->dt_dev, c->nbad, c->stream);
+                         c->lmax, c->dt_dev, c->dt_host_dev, c->nbad, c->stream);
     }
+    c->dt_mapped = c->dt_host != nullptr;
     c->last_stages = 3;
     return check_launch(c, "1D stage");
   }
@@ -441,6 +490,7 @@ int step_device(ws_ctx* c, double* U, double dt) {
       if ((rc = faces(c, s))) return rc;
       if ((rc = update(c, s, U, Us, s == 2 ? U : c->S1, dt))) return rc;
     }
+    c->dt_mapped = c->dt_host != nullptr;
     c->last_stages = 3;
     return WS_OK;
   }
@@ -654,6 +704,7 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
         goto bad;
     }
   }
+  if (!tb) dt_slots.take(&c->dt_host, &c->dt_host_dev);
   if ((rc = dalloc(c, &c->mood_counts, 9)) || (rc = dalloc(c, &c->mask_off_dev, 3))) goto bad;
   if (cudaMemcpy(c->mask_off_dev, c->mask_off, 3 * sizeof(int64_t), cudaMemcpyHostToDevice) != cudaSuccess) {
     rc = fail(c, WS_ECUDA, "copying mask offsets failed");
@@ -761,6 +812,7 @@ int step_graph(ws_ctx* c, double* U) {
       return fail(c, WS_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(e));
     }
     c->graph_U = U;
+    c->graph_mapped = c->dt_mapped;
   }
   CK(c, cudaGraphLaunch(c->graph_exec, c->stream));
   c->last_stages = 3;
@@ -862,8 +914,11 @@ int ws_step(ws_ctx* c, double* U, double dt, double* dt_used) {
   if (rc) return rc;
   if (dt_used) {
     int64_t n = tubes(c) ? c->td.ntubes : 1;
-    CK(c, cudaMemcpyAsync(dt_used, c->dt_dev, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
+    // (a replayed graph writes it as its captured step did)
+    const bool mapped = graph ? c->graph_mapped : !ggraph && c->dt_mapped;
+    if (!mapped) CK(c, cudaMemcpyAsync(dt_used, c->dt_dev, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
+    if (mapped) *dt_used = *c->dt_host;
   }
   if (c->opts.check) {
     unsigned long long nb = 0;
@@ -1164,7 +1219,7 @@ int ws_gate_eval(ws_ctx* c, double* U, uint8_t* smooth) {
   launch_stage2d(c->gd, 3, U, c->Q32, c->Ka, c->Kb, 0.0, c->opts.cfl, c->lmax, c->dt_dev, smooth,
                  smooth + c->mask_off[1], (float)c->opts.eps, c->opts.mood, c->opts.weights, c->nbad, &ga, nullptr,
                  nullptr, 0, false, false, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr,
-                 nullptr, 0, c->stream);
+                 nullptr, 0, nullptr, c->stream);
   return check_launch(c, "gate eval");
 }
 

@@ -233,6 +233,7 @@ struct UpdateArgs {
   double dt_fixed, cfl;
   const unsigned long long* lmax;
   double* dtp;
+  double* dt_host;  // nullable, mapped host memory: receives the step, too
   unsigned long long* nbad;
 };
 
@@ -244,7 +245,10 @@ __global__ void __launch_bounds__(BS) k_update(const __grid_constant__ UpdateArg
   double dt = 0.0;
   if (a.stage == 0) {
     dt = a.dt_fixed > 0.0 ? a.dt_fixed : divide(a.cfl, __longlong_as_double((long long)*a.lmax));
-    if (blockIdx.x == 0 && threadIdx.x == 0) *a.dtp = dt;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      *a.dtp = dt;
+      if (a.dt_host) *a.dt_host = dt;
+    }
   } else if (a.stage > 0) {
     dt = *a.dtp;
   }
@@ -353,8 +357,9 @@ void launch_set_dt(const double*, double dt_fixed, double cfl, const unsigned lo
 
 void launch_update(const GridDev& g, int stage, const double* Un, const double* Us, double* Uout,
                    double* const Fh[3], double* const us[3], double dt_fixed, double cfl,
-                   const unsigned long long* lmax, double* dt_dev, unsigned long long* nbad, cudaStream_t s) {
-  UpdateArgs a{g, stage, Un, Us, Uout, {Fh[0], Fh[1], Fh[2]}, {us[0], us[1], us[2]}, dt_fixed, cfl, lmax, dt_dev, nbad};
+                   const unsigned long long* lmax, double* dt_dev, double* dt_host, unsigned long long* nbad,
+                   cudaStream_t s) {
+  UpdateArgs a{g, stage, Un, Us, Uout, {Fh[0], Fh[1], Fh[2]}, {us[0], us[1], us[2]}, dt_fixed, cfl, lmax, dt_dev, dt_host, nbad};
   const int b = blocks_for(g.ncell);
   switch (g.ndim) {
     case 1: k_update<1><<<b, BS, 0, s>>>(a); break;

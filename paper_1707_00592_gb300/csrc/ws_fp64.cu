@@ -131,6 +131,7 @@ struct LineArgs {
   uint8_t* mask;             // nullable
   unsigned long long* lmax;  // zero before stage 0; stage 2 leaves it zero
   double* dt;
+  double* dt_host;           // nullable, mapped host memory: receives the step, too
   unsigned long long* nbad;  // stage 0 sets it to zero
 };
 
@@ -148,7 +149,10 @@ __global__ void __launch_bounds__(160) k_line(const __grid_constant__ LineArgs a
   if (tid == 0) {
     if (a.stage == 1) {
       dt_sh = a.dt_fixed > 0.0 ? a.dt_fixed : divide_call(a.cfl, __longlong_as_double((long long)*a.lmax));
-      if (blockIdx.x == 0) *a.dt = dt_sh;
+      if (blockIdx.x == 0) {
+        *a.dt = dt_sh;
+        if (a.dt_host) *a.dt_host = dt_sh;
+      }
     } else if (a.stage == 2) {
       dt_sh = *a.dt;
       if (blockIdx.x == 0) *a.lmax = 0ULL;
@@ -300,10 +304,10 @@ void launch_face_fp64(const GridDev& g, const double* Q, double* const Fh[3], do
 }
 
 void launch_line_fp64(const GridDev& g, int stage, double* U, double* L, double* U2, uint8_t* mask, double eps, int mood,
-                      int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt,
+                      int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt, double* dt_host,
                       unsigned long long* nbad, cudaStream_t s) {
   const LineArgs a{g.n[0], stage, g.N, {g.bc[0][0], g.bc[0][1]}, g.dx[0], eps, cfl, dt_fixed, mood, weights, U, L, U2,
-                   mask, lmax, dt, nbad};
+                   mask, lmax, dt, dt_host, nbad};
   switch (scheme_of(eps, weights)) {
     case JS: launch_line<JS>(a, s); break;
     case LITERAL: launch_line<LITERAL>(a, s); break;

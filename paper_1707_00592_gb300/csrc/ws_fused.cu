@@ -193,6 +193,7 @@ struct StageArgs {
   double dt_fixed;    // > 0: use this step; otherwise CFL
   unsigned long long* lmax;  // stage 0: max wave rate (FP64 bits)
   double* dt_out;     // stage 1 (block 0): the dt used
+  double* dt_host;    // nullable, mapped host memory: likewise
   double* U;          // state at t^n; stage 2 replaces it with t^{n+1}
   float* U32;         // FP32 image of U^n (rho, momenta, E - Pi, Gamma, Pi): written in stage 0
   const float* Kin;   // stages 1, 2: accumulated increments
@@ -684,7 +685,10 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
     if (tid == 0) {
       if (a.stage == 1 || a.stage == 2) {  // one FP64 division per CTA
         double d = a.dt_fixed > 0.0 ? a.dt_fixed : (double)a.cfl / __longlong_as_double((long long)*a.lmax);
-        if (a.stage == 1 && MODE != 2 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) *a.dt_out = d;
+        if (a.stage == 1 && MODE != 2 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
+          *a.dt_out = d;
+          if (a.dt_host) *a.dt_host = d;
+        }
         S.dt = f64_to_f32(d);
       }
       // The boxes: this thread, which set the mbarrier up, waits for them; the
@@ -1518,6 +1522,7 @@ static StageArgs stage_args(const GridDev& g, int stage, double* U, float* U32, 
   a.dt_fixed = dt_fixed;
   a.lmax = lmax;
   a.dt_out = dt_out;
+  a.dt_host = nullptr;
   a.U = U;
   a.U32 = U32;
   a.Kin = Kin;
@@ -1580,8 +1585,9 @@ void launch_stage2d(const GridDev& g, int stage, double* U, float* U32, const fl
                     const GateArgs* gate, const int* run_if, unsigned long long* census, int tile, bool pdl,
                     bool img_in, float* img_out, const CUtensorMap* tmk, const CUtensorMap* tmv,
                     unsigned long long* clear0, unsigned long long* clear1, int rows_full, const CUtensorMap* tmk2,
-                    const CUtensorMap* tmv2, int* moving, int stamp, cudaStream_t s) {
+                    const CUtensorMap* tmv2, int* moving, int stamp, double* dt_host, cudaStream_t s) {
   StageArgs a = stage_args(g, stage, U, U32, Kin, Kout, dt_fixed, cfl, lmax, dt_out, eps_rel, mood, weights, nbad);
+  a.dt_host = dt_host;
   a.clear0 = clear0;
   a.clear1 = clear1;
   if (moving && !gate && !census && !run_if && quiet_tiles(g, tile, rows_full)) {
@@ -1788,8 +1794,10 @@ void launch_stage3d(const GridDev& g, int stage, double* U, float* U32, const fl
                     uint8_t* mask_y, uint8_t* mask_z, float eps_rel, int mood, int weights, unsigned long long* nbad,
                     unsigned long long* census, int tile, bool pdl, bool img_in, float* img_out,
                     unsigned long long* clear0, unsigned long long* clear1, const CUtensorMap* tmk,
-                    const CUtensorMap* tmv, const CUtensorMap* tmk2, const CUtensorMap* tmv2, cudaStream_t s) {
+                    const CUtensorMap* tmv, const CUtensorMap* tmk2, const CUtensorMap* tmv2, double* dt_host,
+                    cudaStream_t s) {
   StageArgs a = stage_args(g, stage, U, U32, Kin, Kout, dt_fixed, cfl, lmax, dt_out, eps_rel, mood, weights, nbad);
+  a.dt_host = dt_host;
   a.clear0 = clear0;
   a.clear1 = clear1;
   if (tmk && tmv && !census) {

@@ -108,6 +108,11 @@ struct ws_ctx {
   float* us32[3] = {nullptr, nullptr, nullptr};
   uint8_t* mask = nullptr;      // 3 stages x nmask
   double* dt_dev = nullptr;     // 1 (grid) or ntubes
+  // grids: the step in mapped host memory, written by the step's own kernels
+  // (a copy of eight bytes after the step takes longer than its launches)
+  double* dt_host = nullptr;
+  double* dt_host_dev = nullptr;  // its device address
+  bool dt_mapped = false;         // the last step wrote it
   unsigned long long* lmax = nullptr;  // 1 or ntubes, max wave rate as ordered bits
   unsigned long long* nbad = nullptr;  // inadmissible cells of the last step
   unsigned long long* census = nullptr;  // fused paths: the counts of ws_census_step
@@ -150,6 +155,7 @@ struct ws_ctx {
   bool graph_on = false;
   cudaGraphExec_t graph_exec = nullptr;
   const double* graph_U = nullptr;
+  bool graph_mapped = false;  // the captured step writes dt_host
   // ws_get_mood scratch
   unsigned long long* mood_counts = nullptr;
   int64_t* mask_off_dev = nullptr;
@@ -170,7 +176,8 @@ void launch_set_dt(const double* dt_fixed_or_null, double dt_fixed, double cfl, 
                    double* dt_dev, int64_t n, cudaStream_t s);
 void launch_update(const GridDev& g, int stage, const double* Un, const double* Us, double* Uout,
                    double* const Fh[3], double* const us[3], double dt_fixed, double cfl,
-                   const unsigned long long* lmax, double* dt_dev, unsigned long long* nbad, cudaStream_t s);
+                   const unsigned long long* lmax, double* dt_dev, double* dt_host, unsigned long long* nbad,
+                   cudaStream_t s);
 void launch_mood_count(const uint8_t* mask, int64_t n, int64_t nstage, const int64_t* dir_off, int ndim,
                        unsigned long long* counts, cudaStream_t s);
 
@@ -181,15 +188,15 @@ void launch_face_fp64(const GridDev& g, const double* Q, double* const Fh[3], do
 
 // one RK stage of a 1D grid.  L: nv fields of n values (stage 0 writes them),
 // U2: like U (stage 1 writes it); lmax is zero before stage 0 and after stage 2,
-// dt receives the step in stage 1, stage 0 zeroes nbad
+// dt and (nullable) dt_host receive the step in stage 1, stage 0 zeroes nbad
 void launch_line_fp64(const GridDev& g, int stage, double* U, double* L, double* U2, uint8_t* mask, double eps, int mood,
-                      int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt,
+                      int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt, double* dt_host,
                       unsigned long long* nbad, cudaStream_t s);
 
 // ---- mixed-precision sweep (ws_mixed.cu, FMA allowed) ----
 // the same in mixed precision
 void launch_line_mixed(const GridDev& g, int stage, double* U, float* L, double* U2, uint8_t* mask, float eps_rel, int mood,
-                       int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt,
+                       int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt, double* dt_host,
                        unsigned long long* nbad, cudaStream_t s);
 void launch_prim32(const GridDev& g, const double* U, float* Q, cudaStream_t s);
 void launch_cfl32(const GridDev& g, const float* Q, unsigned long long* lmax, cudaStream_t s);
@@ -236,7 +243,7 @@ void launch_stage2d(const GridDev& g, int stage, double* U, float* U32, const fl
                     const GateArgs* gate, const int* run_if, unsigned long long* census, int tile, bool pdl,
                     bool img_in, float* img_out, const CUtensorMap* tmk, const CUtensorMap* tmv,
                     unsigned long long* clear0, unsigned long long* clear1, int rows_full, const CUtensorMap* tmk2,
-                    const CUtensorMap* tmv2, int* moving, int stamp, cudaStream_t s);
+                    const CUtensorMap* tmv2, int* moving, int stamp, double* dt_host, cudaStream_t s);
 // moving (nullable): 2 x fused2d_max_tiles(g) marks of the tiles that were not
 // quiet (ws_fused.cu) in the step of a stamp; stamp: this step's, from 1, the
 // same for its three stages and never used before with these marks
@@ -266,7 +273,8 @@ void launch_stage3d(const GridDev& g, int stage, double* U, float* U32, const fl
                     uint8_t* mask_y, uint8_t* mask_z, float eps_rel, int mood, int weights, unsigned long long* nbad,
                     unsigned long long* census, int tile, bool pdl, bool img_in, float* img_out,
                     unsigned long long* clear0, unsigned long long* clear1, const CUtensorMap* tmk,
-                    const CUtensorMap* tmv, const CUtensorMap* tmk2, const CUtensorMap* tmv2, cudaStream_t s);
+                    const CUtensorMap* tmv, const CUtensorMap* tmk2, const CUtensorMap* tmv2, double* dt_host,
+                    cudaStream_t s);
 // tmk2, tmv2 (nullable, with tmk and tmv): descriptors of the second pass's
 // boxes (fused2d_encode_map codes 6 and 7); interior z rows of the second
 // pass then load by TMA

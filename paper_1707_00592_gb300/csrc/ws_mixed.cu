@@ -221,6 +221,7 @@ struct LineArgs {
   uint8_t* mask;             // nullable
   unsigned long long* lmax;  // zero before stage 0; stage 2 leaves it zero
   double* dt;
+  double* dt_host;           // nullable, mapped host memory: receives the step, too
   unsigned long long* nbad;  // stage 0 sets it to zero
 };
 
@@ -237,7 +238,10 @@ __global__ void __launch_bounds__(LF) k_line32(const __grid_constant__ LineArgs 
   if (tid == 0) {
     if (a.stage == 1) {
       dt_sh = a.dt_fixed > 0.0 ? a.dt_fixed : fp64::divide(a.cfl, __longlong_as_double((long long)*a.lmax));
-      if (blockIdx.x == 0) *a.dt = dt_sh;
+      if (blockIdx.x == 0) {
+        *a.dt = dt_sh;
+        if (a.dt_host) *a.dt_host = dt_sh;
+      }
     } else if (a.stage == 2) {
       dt_sh = *a.dt;
       if (blockIdx.x == 0) *a.lmax = 0ULL;
@@ -478,10 +482,10 @@ void launch_update_mixed(const GridDev& g, int stage, const double* Un, const do
 }
 
 void launch_line_mixed(const GridDev& g, int stage, double* U, float* L, double* U2, uint8_t* mask, float eps_rel, int mood,
-                       int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt,
+                       int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt, double* dt_host,
                        unsigned long long* nbad, cudaStream_t s) {
   const LineArgs a{g.n[0], stage, g.N, {g.bc[0][0], g.bc[0][1]}, g.dx[0], cfl, dt_fixed, weno_params(eps_rel, weights),
-                   mood, U, L, U2, mask, lmax, dt, nbad};
+                   mood, U, L, U2, mask, lmax, dt, dt_host, nbad};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((a.n + LF - 2) / (LF - 1)));
   cfg.blockDim = dim3(LF);

@@ -136,7 +136,7 @@ extern "C" WS_API int ws_flux_divergence_noalloc(const ws_grid* grid, const ws_o
   double eps = opts->eps > 0.0 ? opts->eps : (opts->weights == WS_W_JS ? 1e-6 : 1e-40);
   launch_prep(g, U, Q, nullptr, nullptr, s);
   launch_face_fp64(g, Q, Fh, us, nullptr, eps, opts->mood, opts->weights, s);
-  launch_update(g, -1, U, U, L, Fh, us, 0.0, 0.0, nullptr, nullptr, nullptr, s);
+  launch_update(g, -1, U, U, L, Fh, us, 0.0, 0.0, nullptr, nullptr, nullptr, nullptr, s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(WS_ECUDA, cudaGetErrorString(e));
   return WS_OK;

@@ -252,47 +252,35 @@ int build_chunks(ws_ctx* c, int config) {
 bool mixed(const ws_ctx* c) { return c->opts.precision == WS_PREC_MIXED; }
 
 // The start of an RHS evaluation of the stage state Us: ghost layers and the
-// primitive cache.  FP64: one launch, which also takes the CFL rate into lmax
+// primitive cache, in one launch that also takes the CFL rate into lmax
 // (nullable, zeroed before) and sets the counter *clear (nullable) to zero.
 int rhs_faces(ws_ctx* c, double* Us, unsigned long long* lmax = nullptr, unsigned long long* clear = nullptr) {
   const GridDev& g = c->gd;
-  if (!mixed(c)) {
-    KScope k(c, WS_K_PRIM);
+  KScope k(c, WS_K_PRIM);
+  if (mixed(c))
+    launch_prep32(g, Us, c->Q32, lmax, clear, c->stream);
+  else
     launch_prep(g, Us, c->Q, lmax, clear, c->stream);
-    return check_launch(c, "ghost/prim");
-  }
-  {
-    KScope k(c, WS_K_GHOST, g.ndim);
-    for (int d = 0; d < g.ndim; ++d) launch_ghost(g, Us, d, c->stream);
-  }
-  {
-    KScope k(c, WS_K_PRIM);
-    launch_prim32(g, Us, c->Q32, c->stream);
-  }
   return check_launch(c, "ghost/prim");
 }
 
 int faces(ws_ctx* c, int stage_slot) {
   const GridDev& g = c->gd;
   uint8_t* mbase = c->mask + (int64_t)stage_slot * c->nmask;
-  if (!mixed(c)) {
-    KScope k(c, WS_K_FACE);
-    uint8_t* const m[3] = {mbase + c->mask_off[0], mbase + c->mask_off[1], mbase + c->mask_off[2]};
+  KScope k(c, WS_K_FACE);
+  uint8_t* const m[3] = {mbase + c->mask_off[0], mbase + c->mask_off[1], mbase + c->mask_off[2]};
+  if (mixed(c))
+    launch_face_mixed(g, c->Q32, c->Fh32, c->us32, m, (float)c->opts.eps, c->opts.mood, c->opts.weights, c->stream);
+  else
     launch_face_fp64(g, c->Q, c->Fh, c->us, m, c->opts.eps, c->opts.mood, c->opts.weights, c->stream);
-    return check_launch(c, "face sweep");
-  }
-  for (int d = 0; d < g.ndim; ++d) {
-    KScope k(c, WS_K_FACE);
-    launch_face_mixed(g, d, c->Q32, c->Fh32[d], c->us32[d], mbase + c->mask_off[d], (float)c->opts.eps, c->opts.mood,
-                      c->opts.weights, c->stream);
-  }
   return check_launch(c, "face sweep");
 }
 
 int update(ws_ctx* c, int stage, const double* Un, const double* Us, double* Uout, double dt = 0.0) {
   KScope k(c, WS_K_UPDATE);
   if (mixed(c))
-    launch_update_mixed(c->gd, stage, Un, Us, Uout, c->Fh32, c->us32, c->Q32, c->dt_dev, c->nbad, c->stream);
+    launch_update_mixed(c->gd, stage, Un, Us, Uout, c->Fh32, c->us32, c->Q32, dt, c->opts.cfl, c->lmax, c->dt_dev,
+                        c->dt_host_dev, c->nbad, c->stream);
   else
     launch_update(c->gd, stage, Un, Us, Uout, c->Fh, c->us, dt, c->opts.cfl, c->lmax, c->dt_dev,
                   c->dt_host_dev, c->nbad, c->stream);
@@ -409,8 +397,8 @@ int step_device(ws_ctx* c, double* U, double dt) {
   int rc;
   c->nbad_last = c->nbad;
   c->dt_mapped = false;
-  // FP64 tubes, a gated step and the general mixed path (the others clear their own counter)
-  if (mixed(c) ? !tubes(c) && (!c->fused || c->learned_on) && g.ndim > 1 : tubes(c))
+  // FP64 tubes and a gated step (the others clear their own counter)
+  if (mixed(c) ? c->learned_on : tubes(c))
     CK(c, cudaMemsetAsync(c->nbad, 0, sizeof(unsigned long long), c->stream));
   if (tubes(c) && mixed(c)) {
     CK(c, cudaMemsetAsync(c->zeroed, 0, c->zeroed_bytes, c->stream));
@@ -478,38 +466,17 @@ int step_device(ws_ctx* c, double* U, double dt) {
     c->last_stages = 3;
     return check_launch(c, "1D stage");
   }
-  if (!mixed(c)) {
-    // three launches per stage.  Stage 0's first zeroes the inadmissible-cell
-    // count and takes the CFL rate, its update derives dt; stage 1's first
-    // zeroes the rate for the next step.
-    for (int s = 0; s < 3; ++s) {
-      double* Us = s == 0 ? U : c->S1;
-      if ((rc = rhs_faces(c, Us, s == 0 && dt <= 0.0 ? c->lmax : nullptr,
-                          s == 0 ? c->nbad : (s == 1 ? c->lmax : nullptr))))
-        return rc;
-      if ((rc = faces(c, s))) return rc;
-      if ((rc = update(c, s, U, Us, s == 2 ? U : c->S1, dt))) return rc;
-    }
-    c->dt_mapped = c->dt_host != nullptr;
-    c->last_stages = 3;
-    return WS_OK;
-  }
+  // Three launches per stage.  Stage 0's first zeroes the inadmissible-cell
+  // count and takes the CFL rate, its update derives dt; stage 1's first zeroes
+  // the rate for the next step.
   for (int s = 0; s < 3; ++s) {
     double* Us = s == 0 ? U : c->S1;
-    if ((rc = rhs_faces(c, Us))) return rc;
-    if (s == 0) {
-      if (dt <= 0.0) {
-        CK(c, cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long), c->stream));
-        KScope k(c, WS_K_CFL);
-        launch_cfl32(g, c->Q32, c->lmax, c->stream);
-      }
-      KScope k(c, WS_K_CFL);
-      launch_set_dt(nullptr, dt, c->opts.cfl, c->lmax, c->dt_dev, 1, c->stream);
-    }
+    if ((rc = rhs_faces(c, Us, s == 0 && dt <= 0.0 ? c->lmax : nullptr, s == 0 ? c->nbad : (s == 1 ? c->lmax : nullptr))))
+      return rc;
     if ((rc = faces(c, s))) return rc;
-    double* Uout = s == 2 ? U : c->S1;
-    if ((rc = update(c, s, U, Us, Uout))) return rc;
+    if ((rc = update(c, s, U, Us, s == 2 ? U : c->S1, dt))) return rc;
   }
+  c->dt_mapped = c->dt_host != nullptr;
   c->last_stages = 3;
   return WS_OK;
 }
@@ -772,7 +739,6 @@ int ws_cfl_dt(ws_ctx* c, double* U, double* dt) {
     CK(c, cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long), c->stream));
     int rc = rhs_faces(c, U, c->lmax);
     if (rc) return rc;
-    if (mixed(c)) launch_cfl32(c->gd, c->Q32, c->lmax, c->stream);
   }
   launch_set_dt(nullptr, 0.0, c->opts.cfl, c->lmax, c->dt_dev, n, c->stream);
   int rc = check_launch(c, "cfl");
@@ -1114,8 +1080,7 @@ int ws_face_samples(ws_ctx* c, double* U, int64_t stride, int64_t max_out, float
   c->img_cur = -1;  // the carried FP32 image no longer follows U
   if (tubes(c) || !mixed(c)) return fail(c, WS_ENOTSUP, "face samples need a mixed-precision grid context");
   const GridDev& g = c->gd;
-  for (int d = 0; d < g.ndim; ++d) launch_ghost(g, U, d, c->stream);
-  launch_prim32(g, U, c->Q32, c->stream);
+  launch_prep32(g, U, c->Q32, nullptr, nullptr, c->stream);
   int64_t out = 0;
   for (int d = 0; d < g.ndim && out < max_out; ++d) {
     launch_face_samples(g, d, c->Q32, stride, out, max_out, feats, labels, (float)c->opts.eps, c->opts.weights,

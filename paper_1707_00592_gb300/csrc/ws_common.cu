@@ -68,41 +68,6 @@ __device__ __forceinline__ void coords(int64_t i, int64_t e0, int64_t e1, int64_
   }
 }
 
-// ---------------------------------------------------------------------------
-// ghost layers of direction d at interior transverse positions
-__global__ void k_ghost(GridDev g, double* __restrict__ U, int d) {
-  int e1 = (d == 0) ? 1 : 0;
-  int e2 = (d == 2) ? 1 : 2;
-  int64_t T1 = g.n[e1], T2 = g.n[e2];
-  int64_t total = T1 * T2 * 2 * NG;
-  int n = g.n[d];
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    int64_t a1 = t % T1;
-    int64_t r = t / T1;
-    int64_t a2 = r % T2;
-    r /= T2;
-    int gI = (int)(r % NG) + 1;
-    int side = (int)(r / NG);
-    int kind = g.bc[d][side];
-    int64_t dst = side == 0 ? (NG - gI) : (NG + n - 1 + gI);
-    int64_t src;
-    if (kind == WS_BC_PERIODIC)
-      src = side == 0 ? (NG + n - gI) : (NG + gI - 1);
-    else if (kind == WS_BC_REFLECTIVE)
-      src = side == 0 ? (NG + gI - 1) : (NG + n - gI);
-    else
-      src = side == 0 ? NG : (NG + n - 1);
-    // unused axes have extent 1 and ghost offset 0, so they add nothing
-    int64_t base = (g.G[e1] + a1) * g.st[e1] + (g.G[e2] + a2) * g.st[e2];
-    int64_t id = base + dst * g.st[d], is = base + src * g.st[d];
-    for (int f = 0; f < g.nv; ++f) {
-      double v = U[f * g.N + is];
-      if (kind == WS_BC_REFLECTIVE && f == 1 + d) v = -v;
-      U[f * g.N + id] = v;
-    }
-  }
-}
-
 // atomicMax of the threads' values
 __device__ __forceinline__ void block_max(unsigned long long b, unsigned long long* out) {
 #pragma unroll
@@ -325,12 +290,6 @@ __global__ void k_mood_count(const uint8_t* __restrict__ mask, int64_t n, int64_
 }
 
 }  // namespace
-
-void launch_ghost(const GridDev& g, double* U, int d, cudaStream_t s) {
-  int e1 = (d == 0) ? 1 : 0, e2 = (d == 2) ? 1 : 2;
-  int64_t total = (int64_t)g.n[e1] * g.n[e2] * 2 * NG;
-  k_ghost<<<blocks_for(total), BS, 0, s>>>(g, U, d);
-}
 
 void launch_prep(const GridDev& g, double* U, double* Q, unsigned long long* lmax, unsigned long long* clear,
                  cudaStream_t s) {

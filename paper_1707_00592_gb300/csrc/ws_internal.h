@@ -165,7 +165,6 @@ struct ws_ctx {
 namespace ws {
 
 // ---- launchers (ws_common.cu, built with -fmad=false) ----
-void launch_ghost(const GridDev& g, double* U, int d, cudaStream_t s);
 // ghost layers of U, primitives Q and (lmax non-null, zeroed before) the CFL
 // rate; clear (nullable): a counter the launch sets to zero
 void launch_prep(const GridDev& g, double* U, double* Q, unsigned long long* lmax, unsigned long long* clear,
@@ -198,15 +197,16 @@ void launch_line_fp64(const GridDev& g, int stage, double* U, double* L, double*
 void launch_line_mixed(const GridDev& g, int stage, double* U, float* L, double* U2, uint8_t* mask, float eps_rel, int mood,
                        int weights, double dt_fixed, double cfl, unsigned long long* lmax, double* dt, double* dt_host,
                        unsigned long long* nbad, cudaStream_t s);
-void launch_prim32(const GridDev& g, const double* U, float* Q, cudaStream_t s);
-void launch_cfl32(const GridDev& g, const float* Q, unsigned long long* lmax, cudaStream_t s);
-void launch_face_mixed(const GridDev& g, int d, const float* Q, float* Fh, float* us, uint8_t* mask, float eps_rel,
-                       int mood, int weights, cudaStream_t s);
+// ghost layers of U, FP32 primitives Q and (lmax non-null, zeroed before) the
+// CFL rate; clear (nullable): a counter the launch sets to zero
+void launch_prep32(const GridDev& g, double* U, float* Q, unsigned long long* lmax, unsigned long long* clear,
+                   cudaStream_t s);
+void launch_face_mixed(const GridDev& g, const float* Q, float* const Fh[3], float* const us[3], uint8_t* const mask[3],
+                       float eps_rel, int mood, int weights, cudaStream_t s);
 void launch_update_mixed(const GridDev& g, int stage, const double* Un, const double* Us, double* Uout,
-                         float* const Fh[3], float* const us[3], const float* Q, const double* dt_dev,
-                         unsigned long long* nbad, cudaStream_t s);
-
-void launch_cfl_u(const GridDev& g, const double* U, unsigned long long* lmax, cudaStream_t s);
+                         float* const Fh[3], float* const us[3], const float* Q, double dt_fixed, double cfl,
+                         const unsigned long long* lmax, double* dt_dev, double* dt_host, unsigned long long* nbad,
+                         cudaStream_t s);
 
 // ---- fused mixed-precision RK stage, 2D and 3D (ws_fused.cu) ----
 struct GateArgs {

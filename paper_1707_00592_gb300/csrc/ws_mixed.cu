@@ -3,10 +3,10 @@
 // cancellation, the sign of the MOOD admissibility test, and the
 // conservative SSP-RK3 accumulation of the FP64 state.
 //
-// Generic form (any dimension): primitive cache in FP32 (k_prim32), one face
-// sweep per direction (k_face32) writing FP32 fluxes, and the update
+// Generic form (any dimension): ghost layers and the primitive cache in FP32
+// (k_prep32), one face sweep (k_face32) writing FP32 fluxes, and the update
 // (k_update_mixed) that forms L(U) in FP32 and accumulates the RK stage in
-// FP64.
+// FP64.  1D steps take k_line32.
 #include <cuda_runtime.h>
 
 #include "face_fp32.cuh"
@@ -50,76 +50,152 @@ __device__ __forceinline__ void cons_to_prim32(const double* U, float* q, float&
   c = fsqrt(sound_speed2(rho, p, Gam, Pi));
 }
 
-template <int NDIM>
-__global__ void k_prim32(GridDev g, const double* __restrict__ U, float* __restrict__ Q) {
-  constexpr int NV = NDIM + 4;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.N; i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t c3[3];
-    c3[0] = i % g.P[0];
-    int64_t r = i / g.P[0];
-    c3[1] = r % g.P[1];
-    c3[2] = r / g.P[1];
-    int out = 0;
-#pragma unroll
-    for (int d = 0; d < NDIM; ++d)
-      if (c3[d] < NG || c3[d] >= NG + g.n[d]) ++out;
-    if (out > 1) continue;
-    double u[NV];
-#pragma unroll
-    for (int f = 0; f < NV; ++f) u[f] = U[f * g.N + i];
-    float q[NV], c;
-    cons_to_prim32<NDIM>(u, q, c);
-#pragma unroll
-    for (int f = 0; f < NV; ++f) Q[f * g.N + i] = q[f];
-    Q[NV * g.N + i] = c;
+// coordinates of linear index i in extents e0, e1 (x fastest), in 32-bit
+// arithmetic where the index allows
+__device__ __forceinline__ void coords(int64_t i, int64_t e0, int64_t e1, int64_t c[3]) {
+  if (i < (1LL << 31)) {
+    const unsigned u = (unsigned)i, r = u / (unsigned)e0, z = r / (unsigned)e1;
+    c[0] = u - r * (unsigned)e0;
+    c[1] = r - z * (unsigned)e1;
+    c[2] = z;
+  } else {
+    c[0] = i % e0;
+    const int64_t r = i / e0;
+    c[1] = r % e1;
+    c[2] = r / e1;
   }
 }
 
+// atomicMax of the threads' wave rates (as doubles: non-negative ones order
+// like their bit patterns, a NaN above +inf)
+__device__ __forceinline__ void block_max(float best, unsigned long long* lmax) {
+  unsigned long long b = (unsigned long long)__double_as_longlong((double)best);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
+    b = v > b ? v : b;
+  }
+  __shared__ unsigned long long sm[32];
+  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (lane == 0) sm[w] = b;
+  __syncthreads();
+  if (w == 0) {
+    b = lane < (int)(blockDim.x >> 5) ? sm[lane] : 0ULL;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
+      b = v > b ? v : b;
+    }
+    if (lane == 0) atomicMax(lmax, b);
+  }
+}
+
+// The start of an RHS evaluation in one launch: ghost layers of U (of the
+// cells with one coordinate outside the interior: the others are never read),
+// FP32 primitives and sound speed of every cell the sweeps read and, with lmax,
+// the CFL rate: max over the interior cells of sum_d (|u_d| + c)/dx_d.
+// clear: a counter set to zero.
 template <int NDIM>
-__global__ void __launch_bounds__(128) k_face32(GridDev g, int d, const float* __restrict__ Q, float* __restrict__ Fh,
-                                                float* __restrict__ us, uint8_t* __restrict__ mask, WenoParams P,
-                                                int mood) {
+__global__ void __launch_bounds__(BS) k_prep32(const __grid_constant__ GridDev g, double* U, float* __restrict__ Q,
+                                               unsigned long long* lmax, unsigned long long* clear) {
+  constexpr int NV = NDIM + 4;
+  if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0ULL;
+  float idx_[3];
+#pragma unroll
+  for (int d = 0; d < NDIM; ++d) idx_[d] = lmax ? (float)(1.0 / g.dx[d]) : 0.0f;
+  float best = 0.0f;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.N; i += (int64_t)gridDim.x * blockDim.x) {
+    int64_t c[3];
+    coords(i, g.P[0], g.P[1], c);
+    int out = 0, flip = -1;
+    int64_t src = i;
+#pragma unroll
+    for (int d = 0; d < NDIM; ++d) {
+      const int64_t x = c[d] - NG;
+      if (x >= 0 && x < g.n[d]) continue;
+      ++out;
+      const int kind = g.bc[d][x < 0 ? 0 : 1];
+      int64_t m = x < 0 ? 0 : g.n[d] - 1;
+      if (kind == WS_BC_PERIODIC) m = x < 0 ? x + g.n[d] : x - g.n[d];
+      if (kind == WS_BC_REFLECTIVE) {
+        m = x < 0 ? -1 - x : 2 * (int64_t)g.n[d] - 1 - x;
+        flip = 1 + d;
+      }
+      src += (m - x) * g.st[d];
+    }
+    if (out > 1) continue;
+    double u[NV];
+#pragma unroll
+    for (int f = 0; f < NV; ++f) {
+      u[f] = U[f * g.N + src];
+      if (f == flip) u[f] = -u[f];
+      if (out) U[f * g.N + i] = u[f];
+    }
+    float q[NV], cs;
+    cons_to_prim32<NDIM>(u, q, cs);
+#pragma unroll
+    for (int f = 0; f < NV; ++f) Q[f * g.N + i] = q[f];
+    Q[NV * g.N + i] = cs;
+    if (lmax && !out) {
+      float lam = 0.0f;
+#pragma unroll
+      for (int d = 0; d < NDIM; ++d) lam = fmaf(fabsf(q[1 + d]) + cs, idx_[d], lam);
+      if (!(lam <= best)) best = lam;  // NaN propagates
+    }
+  }
+  if (lmax) block_max(best, lmax);
+}
+
+struct FaceArgs {
+  GridDev g;
+  const float* Q;
+  float* Fh[3];
+  float* us[3];
+  uint8_t* mask[3];
+  unsigned first[3];  // first CTA of each direction
+  WenoParams P;
+  int mood;
+};
+
+// a thread to a face, the CTAs of one direction after another
+template <int NDIM>
+__global__ void __launch_bounds__(128) k_face32(const __grid_constant__ FaceArgs a) {
   constexpr int NQ = NDIM + 4;
-  const int64_t nf = g.nfaces[d];
-  const int64_t fe0 = g.fe[d][0], fe1 = g.fe[d][1];
-  const int64_t N = g.N;
+  const GridDev& g = a.g;
+  int d = 0;
+#pragma unroll
+  for (int e = 1; e < NDIM; ++e)
+    if (blockIdx.x >= a.first[e]) d = e;
+  const int64_t nf = g.nfaces[d], N = g.N;
+  const int64_t f = (int64_t)(blockIdx.x - a.first[d]) * 128 + threadIdx.x;
+  if (f >= nf) return;
   int fld[NQ];
   fld[0] = 0;
   fld[1] = 1 + d;
-  {
-    int k = 2;
 #pragma unroll
-    for (int e = 0; e < NDIM; ++e)
-      if (e != d) fld[k++] = 1 + e;
-  }
+  for (int m = 2; m < NQ - 3; ++m) fld[m] = m - 2 < d ? m - 1 : m;  // tangential velocities in increasing axis order
   fld[NQ - 3] = 1 + NDIM;
   fld[NQ - 2] = 2 + NDIM;
   fld[NQ - 1] = 3 + NDIM;
+  int64_t c[3];
+  coords(f, g.fe[d][0], g.fe[d][1], c);
+  c[d] -= 1;
   const int64_t sd = g.st[d];
-  for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < nf; f += (int64_t)gridDim.x * blockDim.x) {
-    int64_t c[3];
-    c[0] = f % fe0;
-    int64_t r = f / fe0;
-    c[1] = r % fe1;
-    c[2] = r / fe1;
-    c[d] -= 1;
-    int64_t base = (g.G[0] + c[0]) * g.st[0] + (g.G[1] + c[1]) * g.st[1] + (g.G[2] + c[2]) * g.st[2];
-    float qc[6][NQ], cc[6];
+  const float* q = a.Q + (g.G[0] + c[0]) * g.st[0] + (g.G[1] + c[1]) * g.st[1] + (g.G[2] + c[2]) * g.st[2] - 2 * sd;
+  float qc[6][NQ], cc[6];
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      int64_t idx = base + (j - 2) * sd;
+  for (int j = 0; j < 6; ++j) {
 #pragma unroll
-      for (int m = 0; m < NQ; ++m) qc[j][m] = Q[fld[m] * N + idx];
-      cc[j] = Q[NQ * N + idx];
-    }
-    float Fhat[NQ], ustar;
-    int cl, cr;
-    face<NQ>(qc, cc, P, mood, Fhat, ustar, cl, cr);
-#pragma unroll
-    for (int m = 0; m < NQ; ++m) Fh[fld[m] * nf + f] = Fhat[m];
-    us[f] = ustar;
-    if (mask) mask[f] = (uint8_t)(cl | (cr << 2));
+    for (int m = 0; m < NQ; ++m) qc[j][m] = __ldg(q + fld[m] * N + j * sd);
+    cc[j] = __ldg(q + NQ * N + j * sd);
   }
+  float Fhat[NQ], ustar;
+  int cl, cr;
+  face<NQ>(qc, cc, a.P, a.mood, Fhat, ustar, cl, cr);
+#pragma unroll
+  for (int m = 0; m < NQ; ++m) a.Fh[d][fld[m] * nf + f] = Fhat[m];
+  a.us[d][f] = ustar;
+  if (a.mask[d]) a.mask[d][f] = (uint8_t)(cl | (cr << 2));
 }
 
 // RK stage of one cell from its L in FP32: FP64 accumulation.
@@ -142,61 +218,77 @@ __device__ __forceinline__ bool admissible_cons(const double* o) {
   return rho > 0.0 && Gam > 0.0 && fma(Gam + 1.0, t, -rho * Pi) > 0.0;
 }
 
+// Stage 0 derives the step (dt_fixed, or cfl / *lmax) and leaves it in *dtp for
+// the others; stage -1 writes L itself.
+struct UpdateArgs {
+  GridDev g;
+  int stage;
+  const double *Un, *Us;
+  double* Uout;
+  const float* F[3];
+  const float* u[3];
+  const float* Q;
+  double dt_fixed, cfl;
+  const unsigned long long* lmax;
+  double* dtp;
+  double* dt_host;  // nullable, mapped host memory: receives the step, too
+  unsigned long long* nbad;
+};
+
 template <int NDIM>
-__global__ void k_update_mixed(GridDev g, int stage, const double* Un, const double* Us, double* Uout,
-                               const float* __restrict__ F0, const float* __restrict__ F1,
-                               const float* __restrict__ F2, const float* __restrict__ u0,
-                               const float* __restrict__ u1, const float* __restrict__ u2,
-                               const float* __restrict__ Q, const double* __restrict__ dtp,
-                               unsigned long long* nbad) {
+__global__ void __launch_bounds__(BS) k_update_mixed(const __grid_constant__ UpdateArgs a) {
   constexpr int NV = NDIM + 4;
-  const float* Fd[3] = {F0, F1, F2};
-  const float* ud[3] = {u0, u1, u2};
+  const GridDev& g = a.g;
   float idx_[3];
 #pragma unroll
   for (int d = 0; d < NDIM; ++d) idx_[d] = (float)(1.0 / g.dx[d]);
+  float dt = 1.0f;
+  if (a.stage == 0) {
+    const double s = a.dt_fixed > 0.0 ? a.dt_fixed : fp64::divide(a.cfl, __longlong_as_double((long long)*a.lmax));
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      *a.dtp = s;
+      if (a.dt_host) *a.dt_host = s;
+    }
+    dt = (float)s;
+  } else if (a.stage > 0) {
+    dt = (float)*a.dtp;
+  }
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < g.ncell; t += (int64_t)gridDim.x * blockDim.x) {
-    int64_t a[3];
-    a[0] = t % g.n[0];
-    int64_t r = t / g.n[0];
-    a[1] = r % g.n[1];
-    a[2] = r / g.n[1];
-    int64_t i = (g.G[0] + a[0]) * g.st[0] + (g.G[1] + a[1]) * g.st[1] + (g.G[2] + a[2]) * g.st[2];
-    int64_t fl[3], fr[3];
-    float du[3];
+    int64_t c[3];
+    coords(t, g.n[0], g.n[1], c);
+    const int64_t i = (g.G[0] + c[0]) * g.st[0] + (g.G[1] + c[1]) * g.st[1] + (g.G[2] + c[2]) * g.st[2];
+    int64_t fl[NDIM], fr[NDIM];
+    float du[NDIM];
 #pragma unroll
     for (int d = 0; d < NDIM; ++d) {
-      int64_t b[3] = {a[0], a[1], a[2]};
-      fl[d] = (b[2] * g.fe[d][1] + b[1]) * g.fe[d][0] + b[0];
-      b[d] += 1;
-      fr[d] = (b[2] * g.fe[d][1] + b[1]) * g.fe[d][0] + b[0];
-      du[d] = (ud[d][fr[d]] - ud[d][fl[d]]) * idx_[d];
+      fl[d] = (c[2] * g.fe[d][1] + c[1]) * g.fe[d][0] + c[0];
+      fr[d] = fl[d] + (d == 0 ? 1 : (d == 1 ? g.fe[d][0] : g.fe[d][0] * g.fe[d][1]));
+      du[d] = (a.u[d][fr[d]] - a.u[d][fl[d]]) * idx_[d];
     }
-    float dt = stage >= 0 ? (float)dtp[0] : 1.0f;
     double out[NV];
 #pragma unroll
     for (int f = 0; f < NV; ++f) {
       float L = 0.0f;
 #pragma unroll
       for (int d = 0; d < NDIM; ++d) {
-        int64_t nf = g.nfaces[d];
-        L = fmaf(-(Fd[d][f * nf + fr[d]] - Fd[d][f * nf + fl[d]]), idx_[d], L);
+        const int64_t nf = g.nfaces[d];
+        L = fmaf(-(a.F[d][f * nf + fr[d]] - a.F[d][f * nf + fl[d]]), idx_[d], L);
       }
       if (f >= 2 + NDIM) {
-        float phi = Q[f * g.N + i];
+        float phi = a.Q[f * g.N + i];
         float s = 0.0f;
 #pragma unroll
         for (int d = 0; d < NDIM; ++d) s += du[d];
         L = fmaf(phi, s, L);
       }
-      if (stage < 0)
+      if (a.stage < 0)
         out[f] = (double)L;
       else
-        out[f] = rk_stage(stage, Un[f * g.N + i], Us[f * g.N + i], dt * L);
+        out[f] = rk_stage(a.stage, a.Un[f * g.N + i], a.Us[f * g.N + i], dt * L);
     }
 #pragma unroll
-    for (int f = 0; f < NV; ++f) Uout[f * g.N + i] = out[f];
-    if (stage == 2 && !admissible_cons<NDIM>(out)) atomicAdd(nbad, 1ULL);
+    for (int f = 0; f < NV; ++f) a.Uout[f * g.N + i] = out[f];
+    if (a.stage == 2 && !admissible_cons<NDIM>(out)) atomicAdd(a.nbad, 1ULL);
   }
 }
 
@@ -333,151 +425,51 @@ __global__ void __launch_bounds__(LF) k_line32(const __grid_constant__ LineArgs 
   if (a.stage == 2 && !admissible_cons<1>(out)) atomicAdd(a.nbad, 1ULL);
 }
 
-// max over interior cells of sum_d (|u_d| + c)/dx_d from the FP32 cache
-template <int NDIM>
-__global__ void k_cfl32(GridDev g, const float* __restrict__ Q, unsigned long long* lmax) {
-  constexpr int NV = NDIM + 4;
-  float idx_[3];
-#pragma unroll
-  for (int d = 0; d < NDIM; ++d) idx_[d] = (float)(1.0 / g.dx[d]);
-  float best = 0.0f;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < g.ncell; t += (int64_t)gridDim.x * blockDim.x) {
-    int64_t x = t % g.n[0];
-    int64_t r = t / g.n[0];
-    int64_t y = r % g.n[1];
-    int64_t z = r / g.n[1];
-    int64_t i = (g.G[0] + x) * g.st[0] + (g.G[1] + y) * g.st[1] + (g.G[2] + z) * g.st[2];
-    float c = Q[NV * g.N + i];
-    float lam = 0.0f;
-#pragma unroll
-    for (int d = 0; d < NDIM; ++d) lam = fmaf(fabsf(Q[(1 + d) * g.N + i]) + c, idx_[d], lam);
-    if (!(lam <= best)) best = lam;  // NaN propagates
-  }
-  unsigned long long b = (unsigned long long)__double_as_longlong((double)best);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
-    b = v > b ? v : b;
-  }
-  __shared__ unsigned long long sm[32];
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) sm[w] = b;
-  __syncthreads();
-  if (w == 0) {
-    b = lane < (int)(blockDim.x >> 5) ? sm[lane] : 0ULL;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
-      b = v > b ? v : b;
-    }
-    if (lane == 0) atomicMax(lmax, b);
-  }
-}
-
-// CFL reduction straight from the FP64 state (no primitive cache)
-template <int NDIM>
-__global__ void k_cfl_u(GridDev g, const double* __restrict__ U, unsigned long long* lmax) {
-  constexpr int NV = NDIM + 4;
-  float idx_[3];
-#pragma unroll
-  for (int d = 0; d < NDIM; ++d) idx_[d] = (float)(1.0 / g.dx[d]);
-  float best = 0.0f;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < g.ncell; t += (int64_t)gridDim.x * blockDim.x) {
-    int64_t x = t % g.n[0];
-    int64_t r = t / g.n[0];
-    int64_t y = r % g.n[1];
-    int64_t z = r / g.n[1];
-    int64_t i = (g.G[0] + x) * g.st[0] + (g.G[1] + y) * g.st[1] + (g.G[2] + z) * g.st[2];
-    double u[NV];
-#pragma unroll
-    for (int f = 0; f < NV; ++f) u[f] = U[f * g.N + i];
-    float q[NV], c;
-    cons_to_prim32<NDIM>(u, q, c);
-    float lam = 0.0f;
-#pragma unroll
-    for (int d = 0; d < NDIM; ++d) lam = fmaf(fabsf(q[1 + d]) + c, idx_[d], lam);
-    if (!(lam <= best)) best = lam;
-  }
-  unsigned long long b = (unsigned long long)__double_as_longlong((double)best);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
-    b = v > b ? v : b;
-  }
-  __shared__ unsigned long long sm[32];
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) sm[w] = b;
-  __syncthreads();
-  if (w == 0) {
-    b = lane < (int)(blockDim.x >> 5) ? sm[lane] : 0ULL;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
-      b = v > b ? v : b;
-    }
-    if (lane == 0) atomicMax(lmax, b);
-  }
-}
-
 }  // namespace
 
-void launch_cfl_u(const GridDev& g, const double* U, unsigned long long* lmax, cudaStream_t s) {
-  int b = blocks_for(g.ncell);
-  if (b > 152 * 8) b = 152 * 8;
+void launch_prep32(const GridDev& g, double* U, float* Q, unsigned long long* lmax, unsigned long long* clear,
+                   cudaStream_t s) {
+  const int b = blocks_for(g.N);
   switch (g.ndim) {
-    case 1: k_cfl_u<1><<<b, BS, 0, s>>>(g, U, lmax); break;
-    case 2: k_cfl_u<2><<<b, BS, 0, s>>>(g, U, lmax); break;
-    default: k_cfl_u<3><<<b, BS, 0, s>>>(g, U, lmax); break;
+    case 1: k_prep32<1><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
+    case 2: k_prep32<2><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
+    default: k_prep32<3><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
   }
 }
 
-void launch_cfl32(const GridDev& g, const float* Q, unsigned long long* lmax, cudaStream_t s) {
-  int b = blocks_for(g.ncell);
-  if (b > 152 * 8) b = 152 * 8;
-  switch (g.ndim) {
-    case 1: k_cfl32<1><<<b, BS, 0, s>>>(g, Q, lmax); break;
-    case 2: k_cfl32<2><<<b, BS, 0, s>>>(g, Q, lmax); break;
-    default: k_cfl32<3><<<b, BS, 0, s>>>(g, Q, lmax); break;
+void launch_face_mixed(const GridDev& g, const float* Q, float* const Fh[3], float* const us[3], uint8_t* const mask[3],
+                       float eps_rel, int mood, int weights, cudaStream_t s) {
+  FaceArgs a;
+  a.g = g;
+  a.Q = Q;
+  a.P = weno_params(eps_rel, weights);
+  a.mood = mood;
+  unsigned b = 0;
+  for (int d = 0; d < 3; ++d) {
+    a.Fh[d] = Fh[d];
+    a.us[d] = us[d];
+    a.mask[d] = mask[d];
+    a.first[d] = b;
+    if (d < g.ndim) b += (unsigned)((g.nfaces[d] + 127) / 128);
   }
-}
-
-void launch_prim32(const GridDev& g, const double* U, float* Q, cudaStream_t s) {
-  int b = blocks_for(g.N);
   switch (g.ndim) {
-    case 1: k_prim32<1><<<b, BS, 0, s>>>(g, U, Q); break;
-    case 2: k_prim32<2><<<b, BS, 0, s>>>(g, U, Q); break;
-    default: k_prim32<3><<<b, BS, 0, s>>>(g, U, Q); break;
-  }
-}
-
-void launch_face_mixed(const GridDev& g, int d, const float* Q, float* Fh, float* us, uint8_t* mask, float eps_rel,
-                       int mood, int weights, cudaStream_t s) {
-  WenoParams P = weno_params(eps_rel, weights);
-  int b = blocks_for(g.nfaces[d], 128);
-  switch (g.ndim) {
-    case 1: k_face32<1><<<b, 128, 0, s>>>(g, d, Q, Fh, us, mask, P, mood); break;
-    case 2: k_face32<2><<<b, 128, 0, s>>>(g, d, Q, Fh, us, mask, P, mood); break;
-    default: k_face32<3><<<b, 128, 0, s>>>(g, d, Q, Fh, us, mask, P, mood); break;
+    case 1: k_face32<1><<<b, 128, 0, s>>>(a); break;
+    case 2: k_face32<2><<<b, 128, 0, s>>>(a); break;
+    default: k_face32<3><<<b, 128, 0, s>>>(a); break;
   }
 }
 
 void launch_update_mixed(const GridDev& g, int stage, const double* Un, const double* Us, double* Uout,
-                         float* const Fh[3], float* const us[3], const float* Q, const double* dt_dev,
-                         unsigned long long* nbad, cudaStream_t s) {
-  int b = blocks_for(g.ncell);
+                         float* const Fh[3], float* const us[3], const float* Q, double dt_fixed, double cfl,
+                         const unsigned long long* lmax, double* dt_dev, double* dt_host, unsigned long long* nbad,
+                         cudaStream_t s) {
+  const UpdateArgs a{g, stage, Un, Us, Uout, {Fh[0], Fh[1], Fh[2]}, {us[0], us[1], us[2]}, Q, dt_fixed, cfl, lmax, dt_dev,
+                     dt_host, nbad};
+  const int b = blocks_for(g.ncell);
   switch (g.ndim) {
-    case 1:
-      k_update_mixed<1><<<b, BS, 0, s>>>(g, stage, Un, Us, Uout, Fh[0], Fh[1], Fh[2], us[0], us[1], us[2], Q, dt_dev,
-                                         nbad);
-      break;
-    case 2:
-      k_update_mixed<2><<<b, BS, 0, s>>>(g, stage, Un, Us, Uout, Fh[0], Fh[1], Fh[2], us[0], us[1], us[2], Q, dt_dev,
-                                         nbad);
-      break;
-    default:
-      k_update_mixed<3><<<b, BS, 0, s>>>(g, stage, Un, Us, Uout, Fh[0], Fh[1], Fh[2], us[0], us[1], us[2], Q, dt_dev,
-                                         nbad);
-      break;
+    case 1: k_update_mixed<1><<<b, BS, 0, s>>>(a); break;
+    case 2: k_update_mixed<2><<<b, BS, 0, s>>>(a); break;
+    default: k_update_mixed<3><<<b, BS, 0, s>>>(a); break;
   }
 }
 

@@ -597,7 +597,10 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
           goto bad;
         }
         c->fused = true;
-        c->stage_sched = 1;  // the 3D passes measured faster with plain launches
+        // 32 x 7 tiles with programmatic dependent launch: the fastest of the
+        // eight from 16^3 to 256^3 or within half a percent of it (256^3: 6.54
+        // ms per step, 32 x 15 and plain launches 6.89; 24^3: 50 us against 72)
+        c->stage_tile = 2;
         encode_maps(c);
         c->stage_tma = c->tmap_ok == 0x7u ? 1 : 0;
       }

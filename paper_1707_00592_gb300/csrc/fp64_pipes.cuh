@@ -205,8 +205,8 @@ __device__ __forceinline__ double root(double x) {
   const double s = isqrt(x, rg);
   return in_range(rg) ? s : native_sqrt(x);
 }
-// The same out of line, for kernels that run each division once per thread: a
-// launch of a few warps then waits for less code to be fetched.
+// The same out of line, where a kernel's code is long or runs once per thread:
+// its warps then wait for less of it to be fetched.
 static __device__ __noinline__ double divide_call(double a, double b) { return divide(a, b); }
 static __device__ __noinline__ double root_call(double x) { return root(x); }
 

@@ -367,11 +367,13 @@ int fused_run3(ws_ctx* c, double* U, double dt, const GateArgs* gate, const int*
     const float* Kin = s == 1 ? c->Ka : c->Kb;
     float* Kout = s == 0 ? c->Ka : c->Kb;
     if (g.ndim == 3) {
+      // a census counts by 32 x 15 tiles where no configuration was chosen (their boxes are not the default's)
+      const int tile = census && c->stage_default ? 0 : c->stage_tile;
       const CUtensorMap *tmk = map_of(c, Kin), *tmv = map_of(c, u32);
-      if (!tmk || !tmv) tmk = tmv = nullptr;
+      if (!tmk || !tmv || tile != c->stage_tile) tmk = tmv = nullptr;
       launch_stage3d(g, s, U, u32, Kin, Kout, c->Lp, dt, c->opts.cfl, lmax, c->dt_dev, mb + c->mask_off[0],
                      mb + c->mask_off[1], mb + c->mask_off[2], (float)c->opts.eps, c->opts.mood, c->opts.weights, nbad,
-                     census, c->stage_tile, c->stage_sched == 0, s == 0 && img_in, s == 2 ? img_out : nullptr,
+                     census, tile, c->stage_sched == 0, s == 0 && img_in, s == 2 ? img_out : nullptr,
                      s == 2 ? clr0 : nullptr, s == 2 ? clr1 : nullptr, tmk, tmv, map2_of(c, tmk), map2_of(c, tmv),
                      one_scope ? c->dt_host_dev : nullptr, c->stream);
     } else {
@@ -601,6 +603,7 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
         // eight from 16^3 to 256^3 or within half a percent of it (256^3: 6.54
         // ms per step, 32 x 15 and plain launches 6.89; 24^3: 50 us against 72)
         c->stage_tile = 2;
+        c->stage_default = true;
         encode_maps(c);
         c->stage_tma = c->tmap_ok == 0x7u ? 1 : 0;
       }
@@ -1214,6 +1217,7 @@ static void set_stage_config(ws_ctx* c, int index) {
   c->img_cur = -1;
   const int nl = stage_load_modes(c);
   c->stage_tile = fused_tile_index(c->gd.ndim, index / (2 * nl));
+  c->stage_default = false;
   c->stage_tma = nl == 2 ? (index / 2) % 2 : 0;
   c->stage_sched = index % 2;
   if (c->gd.ndim == 2 && c->stage_tile == 3) set_tail_rows(c);
@@ -1246,6 +1250,7 @@ static int autotune_fused(ws_ctx* c, const double* U, int steps, int* choice) {
   cudaEventCreate(&e1);
   float best = 1e30f;
   int bestk = -1;
+  const bool was_default = c->stage_default;
   const int keep = stage_config_index(c);
   const bool prof = c->prof_on;
   c->prof_on = false;
@@ -1277,6 +1282,7 @@ static int autotune_fused(ws_ctx* c, const double* U, int steps, int* choice) {
   cudaFree(Ut);
   if (rc || bestk < 0) {
     set_stage_config(c, keep);
+    c->stage_default = was_default;
     return rc ? rc : fail(c, WS_ECUDA, "autotune found no configuration");
   }
   set_stage_config(c, bestk);

@@ -79,6 +79,7 @@ struct ws_ctx {
   float* Lp = nullptr;          // fused 3D: x + y part of the divergence (first pass -> second)
   bool fused = false;           // fused mixed-precision stage kernels in use (2D or 3D)
   int stage_tile = 0;           // fused: tile shape of the stage launches (ws_autotune)
+  bool stage_default = false;   // 3D: no configuration was chosen
   int stage_sched = 0;          // fused: 0 stage launches with programmatic dependent launch, 1 plain
                                 // stage launches (ws_autotune)
   int stage_tma = 0;            // fused 2D: 1 interior tiles load image and K as TMA boxes (ws_autotune)

@@ -443,6 +443,7 @@ __device__ __noinline__ void hllc_native(const double (&q)[NQ], int side, double
 template <int NQ, int CH>
 struct FaceSmem {
   double w[CH][NQ][32];  // reconstructed characteristics of the lane pairs of CH chunks
+  int next;              // the first (variable, chunk) no warp has taken yet
 };
 
 // The reconstruction of characteristic variable r on a warp's lane pairs.
@@ -509,15 +510,32 @@ __device__ __forceinline__ void solve(const Faces<NQ, SH>& fc, const double (&w)
   if (!__all_sync(ALL, fine)) hllc_native<NQ>(q, side, out);
 }
 
-// The faces of one CTA of NQ warps: CH chunks of FPW faces, first a variable
-// to a warp, then a chunk to a warp.  at(k) places chunk k, done(k, fc, out,
-// code) takes its results (called by the warps that hold them).  With CH = NQ
-// every warp works in both parts; CH = 1 spreads a short sweep over more SMs.
+// The faces of one CTA of NQ warps: CH chunks of FPW faces, first a variable of
+// a chunk to a warp, then a chunk to a warp.  at(k) places chunk k, done(k, fc,
+// out, code) takes its results (called by the warps that hold them).  With CH =
+// NQ every warp works in both parts; CH = 1 spreads a short sweep over more SMs.
+// Variables differ in work (constant ones have none), so warps take the next
+// (variable, chunk) as they become free; with a fixed variable to each a quarter
+// of their time went into the barrier (512^2 shock-bubble, us per step: 2096
+// fixed, 2035 taken chunk by chunk, 2006 variable by variable, which keeps the
+// warps in the same code; the 48^3 drop 1790, 1747, 1722.  2, 3, 4, 8 and 12
+// warps and chunks to a CTA: 2101, 2089, 2018, 2002, 2064).
 template <int NQ, int CH, Scheme SC, int PI, class At, class Done>
 __device__ __forceinline__ void cta_faces(FaceSmem<NQ, CH>& sm, double eps, int mood, int weights, At at, Done done) {
   const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  if (CH > 1) {
+    if (threadIdx.x == 0) sm.next = CH;
+    __syncthreads();
 #pragma unroll 1
-  for (int k = 0; k < CH; ++k) sm.w[k][r][lane] = reconstruct<NQ, SC, PI>(at(k), r, eps, weights);
+    for (int i = r; i < CH * NQ;) {
+      const int m = i / CH, k = i - m * CH;
+      sm.w[k][m][lane] = reconstruct<NQ, SC, PI>(at(k), m, eps, weights);
+      if (lane == 0) i = atomicAdd(&sm.next, 1);
+      i = __shfl_sync(ALL, i, 0);
+    }
+  } else {
+    sm.w[0][r][lane] = reconstruct<NQ, SC, PI>(at(0), r, eps, weights);
+  }
   __syncthreads();
   // (CH = 1: a different warp from CTA to CTA, so that the SM's sub-partitions share the work)
   const int k = CH == 1 ? (r + (int)(blockIdx.x % NQ)) % NQ : r;

@@ -25,9 +25,10 @@ struct FaceArgs {
 
 // One CTA: CH chunks of FPW consecutive faces of one direction.  24 warps per
 // SM (80 registers): enough to cover the FP64 pipe's latency (96 registers and
-// 18 warps, or 64 registers with spills, measured 2 % slower).  On the 512^2
-// shock-bubble a sweep takes 0.60 ms, the FP64 pipe 80 % busy, against 2.4 ms
-// for one thread per face and native operations.
+// 18 warps, or 64 registers with spills, measured 2 % slower).  Instruction
+// fetches, the barrier and the FP64 pipe share the time: on the 512^2
+// shock-bubble a sweep takes 0.57 ms against 2.4 ms for one thread per face and
+// native operations.
 template <int NDIM, int CH, Scheme SC, int PI>
 __global__ void __launch_bounds__(32 * (NDIM + 4), 24 / (NDIM + 4)) k_face(const __grid_constant__ FaceArgs a) {
   constexpr int NQ = NDIM + 4, H = (NQ + 2) / 2;

@@ -100,6 +100,7 @@ template <int NDIM>
 __global__ void __launch_bounds__(BS) k_prep(const __grid_constant__ GridDev g, double* U, double* __restrict__ Q,
                                              unsigned long long* lmax, unsigned long long* clear) {
   constexpr int NV = NDIM + 4;
+  follow_previous();
   if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0ULL;
   unsigned long long best = 0ULL;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.N; i += (int64_t)gridDim.x * blockDim.x) {
@@ -205,6 +206,7 @@ struct UpdateArgs {
 template <int NDIM>
 __global__ void __launch_bounds__(BS) k_update(const __grid_constant__ UpdateArgs a) {
   constexpr int NV = NDIM + 4;
+  follow_previous();
   const GridDev& g = a.g;
   const double c13 = 1.0 / 3.0, c23 = 2.0 / 3.0;
   double dt = 0.0;
@@ -295,9 +297,9 @@ void launch_prep(const GridDev& g, double* U, double* Q, unsigned long long* lma
                  cudaStream_t s) {
   const int b = blocks_for(g.N);
   switch (g.ndim) {
-    case 1: k_prep<1><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
-    case 2: k_prep<2><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
-    default: k_prep<3><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
+    case 1: launch_following(k_prep<1>, b, BS, s, g, U, Q, lmax, clear); break;
+    case 2: launch_following(k_prep<2>, b, BS, s, g, U, Q, lmax, clear); break;
+    default: launch_following(k_prep<3>, b, BS, s, g, U, Q, lmax, clear); break;
   }
 }
 
@@ -321,9 +323,9 @@ void launch_update(const GridDev& g, int stage, const double* Un, const double* 
   UpdateArgs a{g, stage, Un, Us, Uout, {Fh[0], Fh[1], Fh[2]}, {us[0], us[1], us[2]}, dt_fixed, cfl, lmax, dt_dev, dt_host, nbad};
   const int b = blocks_for(g.ncell);
   switch (g.ndim) {
-    case 1: k_update<1><<<b, BS, 0, s>>>(a); break;
-    case 2: k_update<2><<<b, BS, 0, s>>>(a); break;
-    default: k_update<3><<<b, BS, 0, s>>>(a); break;
+    case 1: launch_following(k_update<1>, b, BS, s, a); break;
+    case 2: launch_following(k_update<2>, b, BS, s, a); break;
+    default: launch_following(k_update<3>, b, BS, s, a); break;
   }
 }
 

@@ -33,6 +33,7 @@ template <int NDIM, int CH, Scheme SC, int PI>
 __global__ void __launch_bounds__(32 * (NDIM + 4), 24 / (NDIM + 4)) k_face(const __grid_constant__ FaceArgs a) {
   constexpr int NQ = NDIM + 4, H = (NQ + 2) / 2;
   __shared__ FaceSmem<NQ, CH> sm;
+  follow_previous();
   int d = 0;
 #pragma unroll
   for (int e = 1; e < NDIM; ++e)
@@ -99,10 +100,10 @@ void launch_faces(FaceArgs a, cudaStream_t s) {
   constexpr int NQ = NDIM + 4;
   unsigned ctas = ctas_of(a, NQ, a.first);
   if (SC != LITERAL && large_sweep(ctas)) {
-    k_face<NDIM, NQ, SC, PIPES><<<ctas, 32 * NQ, 0, s>>>(a);
+    launch_following(k_face<NDIM, NQ, SC, PIPES>, ctas, 32 * NQ, s, a);
   } else {
     ctas = ctas_of(a, 1, a.first);
-    k_face<NDIM, 1, SC, CHAIN><<<ctas, 32 * NQ, 0, s>>>(a);
+    launch_following(k_face<NDIM, 1, SC, CHAIN>, ctas, 32 * NQ, s, a);
   }
 }
 
@@ -143,8 +144,7 @@ __global__ void __launch_bounds__(160) k_line(const __grid_constant__ LineArgs a
   __shared__ double prim[6][C], cons[5][C], flux[6][F];  // cell c of the CTA is cell f0 - 3 + c
   __shared__ double dt_sh;
   __shared__ unsigned long long red[5];
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  follow_previous();
   const int tid = threadIdx.x, n = a.n;
   const int f0 = blockIdx.x * (F - 1);
   if (tid == 0) {
@@ -265,21 +265,10 @@ __global__ void __launch_bounds__(160) k_line(const __grid_constant__ LineArgs a
 template <Scheme SC>
 void launch_line(const LineArgs& a, cudaStream_t s) {
   const unsigned b = (unsigned)((a.n + 5 * FPW - 2) / (5 * FPW - 1)), b1 = (unsigned)((a.n + FPW - 2) / (FPW - 1));
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(160);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (SC != LITERAL && large_sweep(b)) {
-    cfg.gridDim = dim3(b);
-    cudaLaunchKernelEx(&cfg, k_line<5, SC, PIPES>, a);
-  } else {
-    cfg.gridDim = dim3(b1);
-    cudaLaunchKernelEx(&cfg, k_line<1, SC, CHAIN>, a);
-  }
+  if (SC != LITERAL && large_sweep(b))
+    launch_following(k_line<5, SC, PIPES>, b, 160, s, a);
+  else
+    launch_following(k_line<1, SC, CHAIN>, b1, 160, s, a);
 }
 
 }  // namespace

@@ -99,6 +99,7 @@ template <int NDIM>
 __global__ void __launch_bounds__(BS) k_prep32(const __grid_constant__ GridDev g, double* U, float* __restrict__ Q,
                                                unsigned long long* lmax, unsigned long long* clear) {
   constexpr int NV = NDIM + 4;
+  follow_previous();
   if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0ULL;
   float idx_[3];
 #pragma unroll
@@ -161,6 +162,7 @@ struct FaceArgs {
 template <int NDIM>
 __global__ void __launch_bounds__(128) k_face32(const __grid_constant__ FaceArgs a) {
   constexpr int NQ = NDIM + 4;
+  follow_previous();
   const GridDev& g = a.g;
   int d = 0;
 #pragma unroll
@@ -238,6 +240,7 @@ struct UpdateArgs {
 template <int NDIM>
 __global__ void __launch_bounds__(BS) k_update_mixed(const __grid_constant__ UpdateArgs a) {
   constexpr int NV = NDIM + 4;
+  follow_previous();
   const GridDev& g = a.g;
   float idx_[3];
 #pragma unroll
@@ -323,8 +326,7 @@ __global__ void __launch_bounds__(LF) k_line32(const __grid_constant__ LineArgs 
   __shared__ double cons[5][C];
   __shared__ double dt_sh;
   __shared__ float red[LF / 32];
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  follow_previous();
   const int tid = threadIdx.x, n = a.n;
   const int f0 = blockIdx.x * (LF - 1);
   if (tid == 0) {
@@ -431,9 +433,9 @@ void launch_prep32(const GridDev& g, double* U, float* Q, unsigned long long* lm
                    cudaStream_t s) {
   const int b = blocks_for(g.N);
   switch (g.ndim) {
-    case 1: k_prep32<1><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
-    case 2: k_prep32<2><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
-    default: k_prep32<3><<<b, BS, 0, s>>>(g, U, Q, lmax, clear); break;
+    case 1: launch_following(k_prep32<1>, b, BS, s, g, U, Q, lmax, clear); break;
+    case 2: launch_following(k_prep32<2>, b, BS, s, g, U, Q, lmax, clear); break;
+    default: launch_following(k_prep32<3>, b, BS, s, g, U, Q, lmax, clear); break;
   }
 }
 
@@ -453,9 +455,9 @@ void launch_face_mixed(const GridDev& g, const float* Q, float* const Fh[3], flo
     if (d < g.ndim) b += (unsigned)((g.nfaces[d] + 127) / 128);
   }
   switch (g.ndim) {
-    case 1: k_face32<1><<<b, 128, 0, s>>>(a); break;
-    case 2: k_face32<2><<<b, 128, 0, s>>>(a); break;
-    default: k_face32<3><<<b, 128, 0, s>>>(a); break;
+    case 1: launch_following(k_face32<1>, b, 128, s, a); break;
+    case 2: launch_following(k_face32<2>, b, 128, s, a); break;
+    default: launch_following(k_face32<3>, b, 128, s, a); break;
   }
 }
 
@@ -467,9 +469,9 @@ void launch_update_mixed(const GridDev& g, int stage, const double* Un, const do
                      dt_host, nbad};
   const int b = blocks_for(g.ncell);
   switch (g.ndim) {
-    case 1: k_update_mixed<1><<<b, BS, 0, s>>>(a); break;
-    case 2: k_update_mixed<2><<<b, BS, 0, s>>>(a); break;
-    default: k_update_mixed<3><<<b, BS, 0, s>>>(a); break;
+    case 1: launch_following(k_update_mixed<1>, b, BS, s, a); break;
+    case 2: launch_following(k_update_mixed<2>, b, BS, s, a); break;
+    default: launch_following(k_update_mixed<3>, b, BS, s, a); break;
   }
 }
 
@@ -478,16 +480,7 @@ void launch_line_mixed(const GridDev& g, int stage, double* U, float* L, double*
                        unsigned long long* nbad, cudaStream_t s) {
   const LineArgs a{g.n[0], stage, g.N, {g.bc[0][0], g.bc[0][1]}, g.dx[0], cfl, dt_fixed, weno_params(eps_rel, weights),
                    mood, U, L, U2, mask, lmax, dt, dt_host, nbad};
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((a.n + LF - 2) / (LF - 1)));
-  cfg.blockDim = dim3(LF);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_line32, a);
+  launch_following(k_line32, (unsigned)((a.n + LF - 2) / (LF - 1)), LF, s, a);
 }
 
 }  // namespace ws

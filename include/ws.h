@@ -22,9 +22,10 @@
  *    (ws_grid.ntubes > 0) each field is the concatenation of the tubes' padded
  *    segments, tube t on [tube_offsets[t], tube_offsets[t+1]).
  *  - Ghost cells of a state passed to ws_step / ws_flux_divergence /
- *    ws_cfl_dt are scratch: the FP64 path overwrites them from the boundary
- *    conditions, the fused mixed-precision paths apply the boundary
- *    conditions while loading and leave them as they were.  Their contents
+ *    ws_cfl_dt are scratch: the FP64 path and the general mixed one overwrite
+ *    them from the boundary conditions, 1D steps and the fused
+ *    mixed-precision paths apply the boundary conditions while loading and
+ *    leave them as they were.  Their contents
  *    are not inputs and should not be relied on.  Interior cells are only
  *    written by ws_step (and ws_run_host, ws_census_step).
  *  - Work is enqueued on the CUDA stream given to ws_init, in order.  Calls
@@ -364,10 +365,10 @@ WS_API int ws_set_graph(ws_ctx *ctx, int enable);
 /* ---- measurement helpers (not part of the method) ---- */
 
 /* kernel classes for ws_profile_read */
-#define WS_K_GHOST 0   /* ghost layers */
-#define WS_K_PRIM 1    /* conservative -> primitive cache */
-#define WS_K_CFL 2     /* CFL max-reduction and dt */
-#define WS_K_FACE 3    /* face sweep: projection, WENO-IS, MOOD, HLLC */
+#define WS_K_GHOST 0   /* ghost layers (FP64 tubes; on grids part of PRIM) */
+#define WS_K_PRIM 1    /* conservative -> primitive cache, on grids with ghost layers and CFL maximum */
+#define WS_K_CFL 2     /* CFL max-reduction and dt (FP64 tubes) */
+#define WS_K_FACE 3    /* face sweep: projection, WENO-IS, MOOD, HLLC; 1D, fused and mixed tube stages whole */
 #define WS_K_UPDATE 4  /* flux divergence + RK stage */
 #define WS_K_OTHER 5
 #define WS_NKERNEL 8

@@ -78,7 +78,10 @@ __device__ __forceinline__ double quot(double a, double b) {
 // A launch of many CTAs (NQ chunks of faces each) is bound by the pipes, and
 // its products go to the integer pipe; one of few CTAs is bound by the length
 // of its dependency chains: one chunk to a CTA, and products on the FP64 pipe,
-// where their latency is shorter.
+// where their latency is shorter.  The line lies at two CTAs per SM; us per step
+// as small and as large launch: 108^2 (246 CTAs) 234, 241; 122^2 (314) 270, 292;
+// 140^2 (412) 320, 306; 19^3 (195) 282, 324; 22^3 (300) 371, 332; 24^3 (387) 447,
+// 360.
 inline bool large_sweep(unsigned ctas) { return ctas >= 152 * 2; }
 
 __device__ __forceinline__ double fma_exact(double two_k, double a, double b) { return __fma_rn(two_k, a, b); }

@@ -169,7 +169,8 @@ namespace ws {
 // drains; it calls follow_previous() before it touches memory.  What it then
 // releases waits for all of this grid in turn, so a launch never overlaps with
 // more than the end of the one before it.  (Flux divergence of a 641 x 479 grid,
-// three launches: 69.0 us plain, 63.2 so; an FP64 step of 48^3, nine: 1725, 1708.)
+// three launches: 69.0 us plain, 63.2 so; an FP64 step of 48^3, nine: 1725, 1708;
+// of 8 tubes, fourteen: 123, 101.)
 template <class... P, class... A>
 inline void launch_following(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t s, const A&... args) {
   cudaLaunchConfig_t cfg = {};

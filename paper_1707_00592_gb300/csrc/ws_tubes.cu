@@ -24,7 +24,8 @@ inline int blocks_for(int64_t n, int bs = BS) {
   return (int)(b < 1 ? 1 : b);
 }
 
-__global__ void k_tubes_ghost(TubesDev t, double* __restrict__ U) {
+__global__ void k_tubes_ghost(TubesDev t, double* U) {
+  follow_previous();
   int64_t total = t.ntubes * 2 * NG;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
     int64_t tube = k / (2 * NG);
@@ -37,7 +38,10 @@ __global__ void k_tubes_ghost(TubesDev t, double* __restrict__ U) {
   }
 }
 
-__global__ void k_tubes_prim(TubesDev t, const double* __restrict__ U, double* __restrict__ Q) {
+// (U's ghost cells share cache lines with cells that k_tubes_ghost reads: no
+// read-only loads of it in a launch that begins while that one ends)
+__global__ void k_tubes_prim(TubesDev t, const double* U, double* Q) {
+  follow_previous();
   const int64_t N = t.total;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
     double rho = U[i];
@@ -58,6 +62,7 @@ __global__ void k_tubes_prim(TubesDev t, const double* __restrict__ U, double* _
 
 // per-tube max of (|u| + c)/dx: one atomic per warp when the warp lies in one tube
 __global__ void k_tubes_cfl(TubesDev t, const double* __restrict__ Q, unsigned long long* lmax) {
+  follow_previous();
   const int64_t N = t.total;
   for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < N; i0 += (int64_t)gridDim.x * blockDim.x) {
     int64_t i = i0 + threadIdx.x;
@@ -98,6 +103,7 @@ __global__ void __launch_bounds__(160) k_tubes_face(TubesDev t, const double* __
                                                     int mood, int weights) {
   constexpr int H = 3;
   __shared__ FaceSmem<5, CH> sm;
+  follow_previous();
   const int64_t N = t.total;
   const int lane = threadIdx.x & 31, side = lane & 1;
   const int64_t i0 = blockIdx.x * (int64_t)(CH * FPW) + (lane >> 1);
@@ -139,14 +145,15 @@ void tubes_face(const TubesDev& t, const double* Q, double* Fh, double* us, uint
                 int weights, cudaStream_t s) {
   const unsigned b = (unsigned)((t.total + 5 * FPW - 1) / (5 * FPW)), b1 = (unsigned)((t.total + FPW - 1) / FPW);
   if (SC != LITERAL && large_sweep(b))
-    k_tubes_face<5, SC, PIPES><<<b, 160, 0, s>>>(t, Q, Fh, us, mask, eps, mood, weights);
+    launch_following(k_tubes_face<5, SC, PIPES>, b, 160, s, t, Q, Fh, us, mask, eps, mood, weights);
   else
-    k_tubes_face<1, SC, CHAIN><<<b1, 160, 0, s>>>(t, Q, Fh, us, mask, eps, mood, weights);
+    launch_following(k_tubes_face<1, SC, CHAIN>, b1, 160, s, t, Q, Fh, us, mask, eps, mood, weights);
 }
 
 __global__ void k_tubes_update(TubesDev t, int stage, const double* Un, const double* Us, double* Uout,
                                const double* __restrict__ Fh, const double* __restrict__ us,
                                const double* __restrict__ dtp, unsigned long long* nbad) {
+  follow_previous();
   const int64_t N = t.total;
   const double c13 = 1.0 / 3.0, c23 = 2.0 / 3.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
@@ -192,13 +199,13 @@ __global__ void k_tubes_update(TubesDev t, int stage, const double* Un, const do
 }  // namespace
 
 void launch_tubes_ghost(const TubesDev& t, double* U, cudaStream_t s) {
-  k_tubes_ghost<<<blocks_for(t.ntubes * 2 * NG), BS, 0, s>>>(t, U);
+  launch_following(k_tubes_ghost, blocks_for(t.ntubes * 2 * NG), BS, s, t, U);
 }
 void launch_tubes_prim(const TubesDev& t, const double* U, double* Q, cudaStream_t s) {
-  k_tubes_prim<<<blocks_for(t.total), BS, 0, s>>>(t, U, Q);
+  launch_following(k_tubes_prim, blocks_for(t.total), BS, s, t, U, Q);
 }
 void launch_tubes_cfl(const TubesDev& t, const double* Q, unsigned long long* lmax, cudaStream_t s) {
-  k_tubes_cfl<<<blocks_for(t.total), BS, 0, s>>>(t, Q, lmax);
+  launch_following(k_tubes_cfl, blocks_for(t.total), BS, s, t, Q, lmax);
 }
 void launch_tubes_face_fp64(const TubesDev& t, const double* Q, double* Fh, double* us, uint8_t* mask, double eps,
                             int mood, int weights, cudaStream_t s) {
@@ -211,7 +218,7 @@ void launch_tubes_face_fp64(const TubesDev& t, const double* Q, double* Fh, doub
 void launch_tubes_update(const TubesDev& t, int stage, const double* Un, const double* Us, double* Uout,
                          const double* Fh, const double* us, const double* dt_dev, unsigned long long* nbad,
                          cudaStream_t s) {
-  k_tubes_update<<<blocks_for(t.total), BS, 0, s>>>(t, stage, Un, Us, Uout, Fh, us, dt_dev, nbad);
+  launch_following(k_tubes_update, blocks_for(t.total), BS, s, t, stage, Un, Us, Uout, Fh, us, dt_dev, nbad);
 }
 
 }  // namespace ws

@@ -196,6 +196,7 @@ __device__ __forceinline__ long long fix(float v) {
 }
 
 __global__ void k_mlp_acc_out(float* __restrict__ grad, float* __restrict__ loss) {
+  follow_previous();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= NPARAM; i += gridDim.x * blockDim.x) {
     float v = (float)((double)(long long)g_mlp_acc[i] * (1.0 / 281474976710656.0));
     g_mlp_acc[i] = 0ULL;
@@ -259,6 +260,7 @@ __device__ __forceinline__ void dense_relu(const float* W, const float* b, const
 __global__ void __launch_bounds__(GT, 2) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ X,
                                                     const uint8_t* __restrict__ y, int64_t n, float pos_weight,
                                                     float inv_n) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // k_mlp_acc_out, which waits
   extern __shared__ __align__(16) unsigned char grad_raw[];
   GradSmem& S = *reinterpret_cast<GradSmem*>(grad_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -396,6 +398,7 @@ __global__ void __launch_bounds__(GT, 2) k_mlp_grad(const float* __restrict__ pa
 
 __global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
                        const float* __restrict__ g, float lr, float b1, float b2, float eps, float c1, float c2) {
+  follow_previous();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= NPARAM) return;
   float gi = g[i];
@@ -442,7 +445,7 @@ extern "C" WS_API int ws_mlp_grad(const float* params, const float* X, const uin
   if (cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)) != cudaSuccess)
     return WS_ECUDA;
   k_mlp_grad<<<b, GT, sizeof(GradSmem), s>>>(params, X, y, n, pos_weight, 1.0f / (float)n);
-  k_mlp_acc_out<<<(NPARAM + 256) / 256, 256, 0, s>>>(grad, loss);
+  launch_following(k_mlp_acc_out, (NPARAM + 256) / 256, 256, s, grad, loss);
   return cudaGetLastError() == cudaSuccess ? WS_OK : WS_ECUDA;
 }
 
@@ -451,6 +454,7 @@ extern "C" WS_API int ws_mlp_adam(float* params, float* m, float* v, const float
   if (!params || !m || !v || !grad || step < 1) return WS_EINVAL;
   const float b1 = 0.9f, b2 = 0.999f;
   float c1 = 1.0f / (1.0f - powf(b1, (float)step)), c2 = 1.0f / (1.0f - powf(b2, (float)step));
-  k_adam<<<(NPARAM + 255) / 256, 256, 0, (cudaStream_t)stream>>>(params, m, v, grad, lr, b1, b2, 1e-8f, c1, c2);
+  launch_following(k_adam, (NPARAM + 255) / 256, 256, (cudaStream_t)stream, params, m, v, grad, lr, b1, b2, 1e-8f, c1,
+                   c2);
   return cudaGetLastError() == cudaSuccess ? WS_OK : WS_ECUDA;
 }

@@ -320,7 +320,9 @@ WS_API int ws_autotune(ws_ctx *ctx, const double *U, int steps, int *choice);
  * (the default is 14 in 2D: 32 x 15 tile rows closed by 32 x 7 rows, TMA
  * loads, stage launches with programmatic dependent launch -- 12 if the
  * driver cannot describe the buffers for TMA; 6 in 3D: 32 x 7 tiles, TMA
- * loads, programmatic dependent launch -- 4 without TMA).  A TMA candidate
+ * loads, programmatic dependent launch -- 4 without TMA; on 3D grids whose 32
+ * x 15 tiles number at most one and whose 32 x 7 tiles more than one and a
+ * half to an SM 3 or 1: 32 x 15 tiles, plain launches).  A TMA candidate
  * falls back to cell-by-cell loads when the driver refuses a descriptor
  * (ws_get_stage_config then reports loads 0).  WS_EINVAL on a context without
  * fused stages or an index that is not a candidate. */

@@ -602,7 +602,18 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
         // 32 x 7 tiles with programmatic dependent launch: the fastest of the
         // eight from 16^3 to 256^3 or within half a percent of it (256^3: 6.54
         // ms per step, 32 x 15 and plain launches 6.89; 24^3: 50 us against 72)
-        c->stage_tile = 2;
+        // -- but where 32 x 15 tiles leave an SM one CTA at most and 32 x 7 ones
+        // more than one and a half, the larger tile and plain launches: 40 x 22
+        // x 36 74 us against 84, 50 x 28 x 30 76 against 79, 45 x 24 x 30 75
+        // against 77 (30 x 50 x 28, 224 tiles of 32 x 7, 76 either way; 24 x 30 x
+        // 40, 200 tiles, 74 against 68).
+        auto ctas = [&](int ty) {  // of the pass with more tiles
+          const int64_t tx = (g.n[0] + 31) / 32;
+          return std::max(tx * ((g.n[1] + ty - 1) / ty) * g.n[2], tx * ((g.n[2] + ty - 1) / ty) * g.n[1]);
+        };
+        const bool large_tile = ctas(15) <= 152 && ctas(7) > 228;
+        c->stage_tile = large_tile ? 0 : 2;
+        c->stage_sched = large_tile ? 1 : 0;
         c->stage_default = true;
         encode_maps(c);
         c->stage_tma = c->tmap_ok == 0x7u ? 1 : 0;

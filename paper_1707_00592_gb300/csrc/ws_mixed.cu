@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(LF) k_line32(const __grid_constant__ LineArgs 
   __shared__ float prim[6][C], flux[6][LF];  // cell c of the CTA is cell f0 - 3 + c
   __shared__ double cons[5][C];
   __shared__ double dt_sh;
-  __shared__ float red[LF / 32];
+  __shared__ unsigned red[LF / 32];
   follow_previous();
   const int tid = threadIdx.x, n = a.n;
   const int f0 = blockIdx.x * (LF - 1);
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(LF) k_line32(const __grid_constant__ LineArgs 
   }
   if (a.stage != 0) __syncthreads();
   const float idx = (float)(1.0 / a.dx), dt = a.stage != 0 ? (float)dt_sh : 0.0f;
-  float best = 0.0f;
+  unsigned best = 0u;  // the wave rate's bits: non-negative values order like them, a NaN above +inf
   for (int c = tid; c < C && f0 - 3 + c < n + NG; c += LF) {
     const int x = f0 - 3 + c;
     int m = x;
@@ -373,23 +373,17 @@ __global__ void __launch_bounds__(LF) k_line32(const __grid_constant__ LineArgs 
     for (int f = 0; f < 5; ++f) prim[f][c] = q[f];
     prim[5][c] = cs;
     if (a.stage == 0 && x >= 0 && x < n) {
-      const float lam = fmaf(fabsf(q[1]) + cs, idx, 0.0f);
-      if (!(lam <= best)) best = lam;  // NaN propagates
+      best = max(best, __float_as_uint(fmaf(fabsf(q[1]) + cs, idx, 0.0f)));
     }
   }
   if (a.stage == 0 && a.dt_fixed <= 0.0) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float v = __shfl_xor_sync(0xffffffffu, best, o);
-      if (!(v <= best)) best = v;
-    }
+    best = __reduce_max_sync(0xffffffffu, best);
     if ((tid & 31) == 0) red[tid >> 5] = best;
   }
   __syncthreads();
   if (a.stage == 0 && a.dt_fixed <= 0.0 && tid == 0) {
-    for (int w = 1; w < LF / 32; ++w)
-      if (!(red[w] <= best)) best = red[w];
-    atomicMax(a.lmax, (unsigned long long)__double_as_longlong((double)best));
+    for (int w = 1; w < LF / 32; ++w) best = max(best, red[w]);
+    atomicMax(a.lmax, (unsigned long long)__double_as_longlong((double)__uint_as_float(best)));
   }
   if (f0 + tid <= n) {
     float qc[6][5], cc[6];

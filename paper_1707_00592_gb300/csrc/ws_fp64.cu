@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(160) k_line(const __grid_constant__ LineArgs a
       m = x < 0 ? 0 : n - 1;
       if (kind == WS_BC_PERIODIC) m = x < 0 ? x + n : x - n;
       if (kind == WS_BC_REFLECTIVE) {
-        m = x < 0 ? -1 - x : 2 * n - 1 - x;
+        m = x < 0 ? -1 - x : n - 1 - (x - n);
         flip = true;
       }
     }
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(160) k_line(const __grid_constant__ LineArgs a
       if (f >= 3) term = term + phi * du;
       const double L = 0.0 + term;
       if (a.stage == 0) {
-        a.L[f * n + x] = L;
+        a.L[(int64_t)f * n + x] = L;
         continue;
       }
       const double un = a.U[f * a.N + NG + x];

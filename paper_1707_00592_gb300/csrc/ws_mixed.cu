@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(LF) k_line32(const __grid_constant__ LineArgs 
       m = x < 0 ? 0 : n - 1;
       if (kind == WS_BC_PERIODIC) m = x < 0 ? x + n : x - n;
       if (kind == WS_BC_REFLECTIVE) {
-        m = x < 0 ? -1 - x : 2 * n - 1 - x;
+        m = x < 0 ? -1 - x : n - 1 - (x - n);
         flip = true;
       }
     }
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(LF) k_line32(const __grid_constant__ LineArgs 
     float L = fmaf(-(flux[f][tid + 1] - flux[f][tid]), idx, 0.0f);
     if (f >= 3) L = fmaf(prim[f][tid + 3], 0.0f + du, L);
     if (a.stage == 0)
-      a.L[f * n + x] = L;
+      a.L[(int64_t)f * n + x] = L;
     else
       out[f] = rk_stage(a.stage, a.U[f * a.N + NG + x], cons[f][tid + 3], dt * L);
   }

@@ -704,15 +704,13 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
   auto quiet_end = [&]() {
     float* out = a.stage == 0 || a.stage == 1 ? a.Kout : a.img_out;
     if (out) {
-      float v[NQ];
-#pragma unroll
-      for (int m = 0; m < NQ; ++m) v[m] = a.stage == 2 ? a.U32[m * N32 + idx32(y0, x0)] : 0.0f;
       for (int c = tid; c < TX * TY; c += NT) {
         const int j = c / TX, i = c - j * TX;
         if (x0 + i >= nx || y0 + j >= n1) continue;
         const int64_t gf = idx32(y0 + j, x0 + i);
+        // (a cell keeps its own image: cells of one pressure may differ in energy)
 #pragma unroll
-        for (int m = 0; m < NQ; ++m) out[m * N32 + gf] = v[m];
+        for (int m = 0; m < NQ; ++m) out[m * N32 + gf] = a.stage == 2 ? a.U32[m * N32 + gf] : 0.0f;
       }
     }
     for (int f = tid; f < T::NFP; f += NT) {

@@ -342,7 +342,7 @@ int fused_run3(ws_ctx* c, double* U, double dt, const GateArgs* gate, const int*
   float* u32 = c->Q32;
   bool img_in = false;
   float* img_out = nullptr;
-  if (c->resident && one_scope) {
+  if (c->resident && one_scope && !c->capturing) {
     if (c->img_cur >= 0 && c->img_U == U) {
       u32 = c->img[c->img_cur];
       img_in = true;
@@ -820,6 +820,14 @@ int gated_step_graph(ws_ctx* c, double* U, double dt) {
         if (g) cudaGraphDestroy(g);
       }
     } guard{g};
+    // captured stages take the context's own counters and clear them, and
+    // leave the tiles' marks and the carried image alone: a replay repeats
+    // the slots, the stamp and the buffers of its capture
+    struct CaptureGuard {
+      ws_ctx* c;
+      explicit CaptureGuard(ws_ctx* c) : c(c) { c->capturing = true; }
+      ~CaptureGuard() { c->capturing = false; }
+    } capture(c);
     cudaGraphConditionalHandle cond;
     CK(c, cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault));
     // main part: the gated stages and the decision

@@ -283,7 +283,9 @@ WS_API int ws_gate_stats(ws_ctx *ctx, double out[6]);
  * for `steps` CFL steps (after one warm-up step) on a scratch copy of U
  * (DEVICE; U itself is not modified), in two rounds over the candidates; a
  * candidate's time is its faster round.  Every candidate gives bit-identical
- * results; only the time differs.
+ * results; only the time differs.  Fused stages are timed with every face
+ * evaluated, also where U is at rest, and the configuration in use stays
+ * where no other is faster by more than the rounds differ.
  *  - Fused 2D/3D mixed-precision stages (learned gate off): the tile of cells
  *    a CTA owns and its thread count -- 32 x 15 cells on 512 threads (two CTAs
  *    per SM), 32 x 31 on 1024 (one CTA per SM; 2D only: with 7 fields its

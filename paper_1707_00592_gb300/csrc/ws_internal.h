@@ -90,6 +90,7 @@ struct ws_ctx {
   unsigned long long* chain = nullptr;
   int64_t chain_n = 0;
   unsigned long long* nbad_last = nullptr;
+  bool tuning = false;          // ws_autotune times the steps (no quiet tiles)
   bool capturing = false;       // a step is being captured into a graph (no chained slots)
   // fused 2D: TMA descriptors of Ka, Kb, Q32, img[0], img[1] for the current
   // tile shape, and [5..9] the same for the closing rows of tile 3; tmap_ok

@@ -390,11 +390,12 @@ __device__ __forceinline__ bool hllc_pair(const double (&q)[NQ], int side, doubl
   const double po = partner(p), ko = partner(ks), mo = partner(ms);
   const double num = (((side ? p - po : po - p)) + (side ? ko : ks)) - (side ? ks : ko);
   const double Ss = quot<PI>(num, side ? mo - ms : ms - mo);
+  auto small = [](double x) { return (hi_of(x) & 0x7fffffffu) < ((1023u + 150u) << 20); };
+  if (!(small(S) && small(Ss))) rg = 0u;  // no product below exceeds 2^700
   // Eq. (flux-function), D* = (0, 1, 0.., S*, 0, 0), and Eq. (velocities)
   const double SP = mul<PI>(S, p + mul<PI>(ms, Ss - un, rg), rg), SPS = mul<PI>(SP, Ss, rg);
   const double dS = S - Ss;
   // only the side that S* selects contributes if the other's flux is finite
-  auto small = [](double x) { return (hi_of(x) & 0x7fffffffu) < ((1023u + 150u) << 20); };
   const bool ok = moderate && small(S) && small(Ss) && small(E) && small(dS) && (hi_of(dS) & 0x7fffffffu) > ((1023u - 150u) << 20) &&
             !is_zero(Ss);
   const unsigned b = __ballot_sync(ALL, ok);

@@ -173,10 +173,12 @@ namespace ws {
 // three launches: 69.0 us plain, 63.2 so; an FP64 step of 48^3, nine: 1725, 1708;
 // of 8 tubes, fourteen: 123, 101.)
 template <class... P, class... A>
-inline void launch_following(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t s, const A&... args) {
+inline void launch_following_smem(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                                  const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -184,6 +186,10 @@ inline void launch_following(void (*kernel)(P...), unsigned grid, unsigned block
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <class... P, class... A>
+inline void launch_following(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t s, const A&... args) {
+  launch_following_smem(kernel, grid, block, 0, s, args...);
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void follow_previous() {

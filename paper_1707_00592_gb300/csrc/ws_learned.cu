@@ -187,8 +187,13 @@ __global__ void k_mlp_forward(const float* __restrict__ params, const float* __r
 // and blocks come in, and a gradient is the same on every run.  Each
 // contribution is rounded to the unit once (|contributions| < 3e4).
 constexpr float kFixScale = 281474976710656.0f;  // 2^48
-// the sums; [NPARAM]: the loss.  Zero between calls: k_mlp_acc_out leaves it so
+// the sums; [NPARAM]: the loss.  Each call sets them to zero first
 __device__ unsigned long long g_mlp_acc[NPARAM + 1];
+
+__global__ void k_mlp_acc_zero() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // k_mlp_grad, which waits before it adds
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= NPARAM; i += gridDim.x * blockDim.x) g_mlp_acc[i] = 0ULL;
+}
 
 __device__ __forceinline__ long long fix(float v) {
   float s = fminf(fmaxf(v * kFixScale, -9.0e18f), 9.0e18f);  // exact scaling by a power of two
@@ -199,7 +204,6 @@ __global__ void k_mlp_acc_out(float* __restrict__ grad, float* __restrict__ loss
   follow_previous();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= NPARAM; i += gridDim.x * blockDim.x) {
     float v = (float)((double)(long long)g_mlp_acc[i] * (1.0 / 281474976710656.0));
-    g_mlp_acc[i] = 0ULL;
     if (i < NPARAM)
       grad[i] = v;
     else
@@ -381,6 +385,7 @@ __global__ void __launch_bounds__(GT, 2) k_mlp_grad(const float* __restrict__ pa
     }
     __syncthreads();  // the next tile takes the arrays
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the sums are zero
   auto add = [](int i, long long v) {
     if (v != 0) atomicAdd(&g_mlp_acc[i], (unsigned long long)v);
   };
@@ -444,7 +449,10 @@ extern "C" WS_API int ws_mlp_grad(const float* params, const float* X, const uin
   if (b > 152 * 2) b = 152 * 2;  // two CTAs per SM
   if (cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)) != cudaSuccess)
     return WS_ECUDA;
-  k_mlp_grad<<<b, GT, sizeof(GradSmem), s>>>(params, X, y, n, pos_weight, 1.0f / (float)n);
+  // (k_mlp_acc_zero begins when everything before it has ended, so k_mlp_grad
+  // may read its inputs while that one runs)
+  k_mlp_acc_zero<<<(NPARAM + 256) / 256, 256, 0, s>>>();
+  launch_following_smem(k_mlp_grad, b, GT, sizeof(GradSmem), s, params, X, y, n, pos_weight, 1.0f / (float)n);
   launch_following(k_mlp_acc_out, (NPARAM + 256) / 256, 256, s, grad, loss);
   return cudaGetLastError() == cudaSuccess ? WS_OK : WS_ECUDA;
 }

@@ -243,8 +243,8 @@ int build_chunks(ws_ctx* c, int config) {
   c->lmax = z + 1;
   c->counters = reinterpret_cast<unsigned*>(z + 1 + nt);
   c->nbad_last = nullptr;
-  CK(c, cudaMemset(z, 0, c->zeroed_bytes));
-  CK(c, cudaMemcpy(c->chunks, items.data(), n * sizeof(TubeItem), cudaMemcpyHostToDevice));
+  CK(c, cudaMemsetAsync(z, 0, c->zeroed_bytes, c->stream));
+  CK(c, cudaMemcpyAsync(c->chunks, items.data(), n * sizeof(TubeItem), cudaMemcpyHostToDevice, c->stream));
   c->nchunks = n;
   c->tube_config = config;
   return WS_OK;
@@ -576,7 +576,7 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
         if ((rc = dalloc(c, &c->Ka, (int64_t)g.nv * g.N32)) || (rc = dalloc(c, &c->Kb, (int64_t)g.nv * g.N32)) ||
             (rc = dalloc(c, &c->census, 4)) || (rc = dalloc(c, &c->moving, 2 * fused2d_max_tiles(g))))
           goto bad;
-        if (cudaMemset(c->moving, 0, 2 * sizeof(int) * fused2d_max_tiles(g)) != cudaSuccess) {
+        if (cudaMemsetAsync(c->moving, 0, 2 * sizeof(int) * fused2d_max_tiles(g), c->stream) != cudaSuccess) {
           rc = fail(c, WS_ECUDA, "cannot clear the tile marks");
           goto bad;
         }
@@ -620,7 +620,7 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
       }
       if (c->fused) {  // slots of consecutive plain steps, cleared once here
         if ((rc = dalloc(c, &c->chain, 4))) goto bad;
-        if (cudaMemset(c->chain, 0, 4 * sizeof(unsigned long long)) != cudaSuccess) {
+        if (cudaMemsetAsync(c->chain, 0, 4 * sizeof(unsigned long long), c->stream) != cudaSuccess) {
           rc = fail(c, WS_ECUDA, "cannot clear the step counters");
           goto bad;
         }
@@ -674,8 +674,10 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
         (rc = dalloc(c, &c->us[0], total)) || (rc = dalloc(c, &c->off_dev, nt + 1)) ||
         (rc = dalloc(c, &c->cell_tube, total)))
       goto bad;
-    if (cudaMemcpy(c->off_dev, off.data(), sizeof(int64_t) * (nt + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(c->cell_tube, ct.data(), sizeof(int) * total, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (cudaMemcpyAsync(c->off_dev, off.data(), sizeof(int64_t) * (nt + 1), cudaMemcpyHostToDevice, c->stream) !=
+            cudaSuccess ||
+        cudaMemcpyAsync(c->cell_tube, ct.data(), sizeof(int) * total, cudaMemcpyHostToDevice, c->stream) !=
+            cudaSuccess) {
       rc = fail(c, WS_ECUDA, "copying tube offsets failed");
       goto bad;
     }
@@ -690,16 +692,20 @@ int ws_init(const ws_grid* grid, const ws_opts* opts, void* stream, ws_ctx** out
   }
   if (!tb) dt_slots.take(&c->dt_host, &c->dt_host_dev);
   if ((rc = dalloc(c, &c->mood_counts, 9)) || (rc = dalloc(c, &c->mask_off_dev, 3))) goto bad;
-  if (cudaMemcpy(c->mask_off_dev, c->mask_off, 3 * sizeof(int64_t), cudaMemcpyHostToDevice) != cudaSuccess) {
+  // what a context starts with is set on its own stream: one that does not
+  // wait for the legacy stream could step before, or be overwritten after
+  // (the copies' sources are pageable, staged before the calls return)
+  if (cudaMemcpyAsync(c->mask_off_dev, c->mask_off, 3 * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream) !=
+      cudaSuccess) {
     rc = fail(c, WS_ECUDA, "copying mask offsets failed");
     goto bad;
   }
-  if (cudaMemset(c->lmax, 0, sizeof(unsigned long long)) != cudaSuccess) {  // FP64 grid steps leave it at zero
+  if (cudaMemsetAsync(c->lmax, 0, sizeof(unsigned long long), c->stream) != cudaSuccess) {  // FP64 grid steps leave it at zero
     rc = fail(c, WS_ECUDA, "cudaMemset failed");
     goto bad;
   }
   // tube masks hold one byte per padded cell; the bytes that carry no face stay 0xff
-  if (cudaMemset(c->mask, tb ? 0xff : 0, 3 * c->nmask) != cudaSuccess) {
+  if (cudaMemsetAsync(c->mask, tb ? 0xff : 0, 3 * c->nmask, c->stream) != cudaSuccess) {
     rc = fail(c, WS_ECUDA, "cudaMemset failed");
     goto bad;
   }

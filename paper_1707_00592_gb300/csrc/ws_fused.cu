@@ -709,8 +709,13 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
         if (x0 + i >= nx || y0 + j >= n1) continue;
         const int64_t gf = idx32(y0 + j, x0 + i);
         // (a cell keeps its own image: cells of one pressure may differ in energy)
+        if (a.stage == 2) {
 #pragma unroll
-        for (int m = 0; m < NQ; ++m) out[m * N32 + gf] = a.stage == 2 ? a.U32[m * N32 + gf] : 0.0f;
+          for (int m = 0; m < NQ; ++m) out[m * N32 + gf] = a.U32[m * N32 + gf];
+        } else {
+#pragma unroll
+          for (int m = 0; m < NQ; ++m) out[m * N32 + gf] = 0.0f;
+        }
       }
     }
     for (int f = tid; f < T::NFP; f += NT) {
@@ -726,7 +731,7 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
   };
   if constexpr (QUIET) {
     if (a.stage != 0) {
-      bool quiet = true;
+      bool quiet = fabsf(S.dt) < INFINITY;  // a step that is not finite reaches every cell
 #pragma unroll
       for (int k = 0; k < 5; ++k) quiet = quiet && S.moved[k] != a.stamp;
       if (quiet) {

@@ -19,7 +19,8 @@
 // stage 1 works through the chunks that move and those beside them, stage 2
 // also through the next ones, and neither touches the rest (a chunk's halo
 // lies in the chunks beside it).  The results are those of evaluating
-// everything, bit for bit.
+// everything, bit for bit; the chunks of a tube whose step is not finite are
+// all worked through (list_tube).
 //
 // While a CTA works on an item, its first thread fetches the next one's
 // description and CFL rate step by step with asynchronous copies, so that no
@@ -89,6 +90,28 @@ __device__ __forceinline__ bool quiet_state(float rho, float u, float p, float G
          fmaf(G + 1.0f, p, Pi) > 1e-4f * ((G + 1.0f) * (fabsf(p) + rho * c * fabsf(u)) + fabsf(Pi));
 }
 
+// Stage 1 of tube t with a step that is not finite: the step reaches every
+// cell, those of chunks that stage 0 left out too.  In stage 1 their states are
+// not numbers (0 times the step): both sides of their faces take the last resort
+// of the MOOD cascade, and the increments don't matter any more; stage 2 works
+// through them.
+__device__ __noinline__ void list_tube(const TubeArgs& a, int64_t t, int chunk) {
+  int64_t lo = 0, hi = a.w.nitems;  // the tube's first item
+  while (lo < hi) {
+    const int64_t m = (lo + hi) / 2;
+    if (a.w.items[m].tube < t)
+      lo = m + 1;
+    else
+      hi = m;
+  }
+  for (int64_t j = lo; j < a.w.nitems && a.w.items[j].tube == t; ++j) {
+    const TubeItem it = a.w.items[j];
+    if (a.mask && a.w.listed[j] == 0)
+      for (int f = 0; f <= min(chunk, it.len - it.c0); ++f) a.mask[it.off + NG + it.c0 + f - 1] = a.mood ? 2 | (2 << 2) : 0;
+    if (atomicExch(&a.w.listed[a.w.nitems + j], 1) == 0) a.w.list[a.w.nitems + atomicAdd(&a.w.counters[4], 1u)] = it;
+  }
+}
+
 template <int CH, int NTH>
 __global__ void __launch_bounds__(NTH, 1024 / NTH) k_tube_stage(const __grid_constant__ TubeArgs a) {  // 64 registers
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -101,8 +124,11 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) k_tube_stage(const __grid_con
   const unsigned nitems = a.stage == 0 ? (unsigned)a.w.nitems : a.w.counters[2 + a.stage];
   unsigned* counter = a.w.counters + a.stage;
   if (a.stage == 1)  // the steps of all tubes
-    for (int64_t t = blockIdx.x * (int64_t)NTH + tid; t < a.t.ntubes; t += (int64_t)gridDim.x * NTH)
-      a.dt_out[t] = a.dt_fixed > 0.0 ? a.dt_fixed : (double)a.cfl / __longlong_as_double((long long)a.lmax[t]);
+    for (int64_t t = blockIdx.x * (int64_t)NTH + tid; t < a.t.ntubes; t += (int64_t)gridDim.x * NTH) {
+      const double d = a.dt_fixed > 0.0 ? a.dt_fixed : (double)a.cfl / __longlong_as_double((long long)a.lmax[t]);
+      a.dt_out[t] = d;
+      if (!(fabsf(f64_to_f32(d)) < INFINITY)) list_tube(a, t, CH);
+    }
   // thread 0: makes the item in S.next the current one
   auto take = [&](unsigned k) {
     S.more = k < nitems;

@@ -154,7 +154,7 @@ struct Smem {
     // phase A before the own cells' arrays are filled
     float kbox[MODE == 2 ? NQ_ : 1][MODE == 2 ? HY : 1][MODE == 2 ? T::QP : 1];
   };
-  unsigned long long red[NT / 32];  // per-warp CFL maxima
+  unsigned red[NT / 32];            // per-warp CFL maxima (FP32 bits)
   unsigned long long mbar;          // completion of the TMA loads
   float dt;                         // the step, broadcast from thread 0
   int moved[5];                     // quiet tiles: marks of this tile and its neighbours
@@ -766,7 +766,7 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
   if (CACHE && (a.stage == 2 || MODE == 2)) own_copies(a.stage == 2, !(MODE == 2 && tma));
   const float dt = (a.stage == 1 || a.stage == 2) ? S.dt : 0.0f;
   const float coef = a.stage == 0 ? 0.0f : (a.stage == 1 ? dt : 0.25f * dt);
-  float lam_max = 0.0f;
+  unsigned lam_max = 0u;  // the wave rate's bits: non-negative values order like them, a NaN above +inf
   float p_own = -1.0f;  // QUIET, stage 0: a pressure of this thread's cells
 
   if (LEARNED) {  // this thread's drift sums (only it touches them until after phase B)
@@ -828,7 +828,7 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
       if (a.stage == 0 && MODE != 2 && ownc) {
         float lam = fmaf(fabsf(vel[0]) + c, a.idx, (fabsf(vel[1]) + c) * a.idy);
         if (ND == 3) lam = fmaf(fabsf(vel[ND - 1]) + c, a.idz, lam);
-        if (!(lam <= lam_max)) lam_max = lam;  // NaN propagates
+        lam_max = max(lam_max, __float_as_uint(lam));
       }
     };
     if (tma && MODE == 2) {  // the boxes have landed (barrier above)
@@ -950,21 +950,16 @@ __device__ __forceinline__ void stage_body(const StageArgs& a, const int trow, c
     }
   }
   if (a.stage == 0 && MODE != 2) {
-    unsigned long long b = (unsigned long long)__double_as_longlong(f32_to_f64(lam_max));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
-      b = v > b ? v : b;
-    }
-    if ((tid & 31) == 0) S.red[tid >> 5] = b;
+    lam_max = __reduce_max_sync(0xffffffffu, lam_max);
+    if ((tid & 31) == 0) S.red[tid >> 5] = lam_max;
   }
   if (QUIET && a.stage == 0 && tid == 32) cp_async_wait_all();
   __syncthreads();
   if (a.stage == 0 && MODE != 2 && tid == 0) {
-    unsigned long long b = 0;
+    unsigned b = 0;
 #pragma unroll
-    for (int w = 0; w < NT / 32; ++w) b = S.red[w] > b ? S.red[w] : b;
-    if (b) atomicMax(a.lmax, b);
+    for (int w = 0; w < NT / 32; ++w) b = max(b, S.red[w]);
+    if (b) atomicMax(a.lmax, (unsigned long long)__double_as_longlong(f32_to_f64(__uint_as_float(b))));
   }
   if constexpr (QUIET) {
     if (a.stage == 0) {  // mark the tile unless its cells hold one state

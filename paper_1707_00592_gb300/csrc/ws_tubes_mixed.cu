@@ -49,7 +49,7 @@ struct TSmem {
   TubeItem now;
   int more;                      // now holds an item
   float dt;
-  unsigned long long red[32];
+  unsigned red[32];
 };
 
 struct TubeArgs {
@@ -165,7 +165,8 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) k_tube_stage(const __grid_con
     const int nc = min(CH, len - c0);  // cells of this chunk
     const float idx = (float)len;      // 1/dx, dx = 1/len
     // ---- phase A ----
-    float lam = 0.0f, p_own = -1.0f;
+    float p_own = -1.0f;
+    unsigned lam = 0u;  // the wave rate's bits: non-negative values order like them, a NaN above +inf
     for (int h = tid; h < nc + 2 * NG; h += NTH) {
       int gc = c0 + h - NG;  // tube-local interior index
       int mc = gc < 0 ? 0 : (gc >= len ? len - 1 : gc);
@@ -205,24 +206,18 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) k_tube_stage(const __grid_con
       S.q[5][h] = c;
       p_own = p;
       if (a.stage == 0 && h >= NG && h < NG + nc) {
-        float l = (fabsf(u) + c) * idx;
-        if (!(l <= lam)) lam = l;
+        lam = max(lam, __float_as_uint((fabsf(u) + c) * idx));
       }
     }
     if (a.stage == 0) {
-      unsigned long long b = (unsigned long long)__double_as_longlong(f32_to_f64(lam));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
-        b = v > b ? v : b;
-      }
-      if ((tid & 31) == 0) S.red[tid >> 5] = b;
+      lam = __reduce_max_sync(0xffffffffu, lam);
+      if ((tid & 31) == 0) S.red[tid >> 5] = lam;
       // one pressure in every warp: worth a look at all cells
       bool quiet = __syncthreads_and(p_own == __shfl_sync(0xffffffffu, p_own, 0) || p_own == -1.0f);
       if (tid == 0) {
-        unsigned long long r = 0;
-        for (int w = 0; w < NTH / 32; ++w) r = S.red[w] > r ? S.red[w] : r;
-        if (r) atomicMax(&a.lmax[tube], r);
+        unsigned r = 0;
+        for (int w = 0; w < NTH / 32; ++w) r = max(r, S.red[w]);
+        if (r) atomicMax(&a.lmax[tube], (unsigned long long)__double_as_longlong(f32_to_f64(__uint_as_float(r))));
         fetch_item(nxt);
       }
       if (quiet) {

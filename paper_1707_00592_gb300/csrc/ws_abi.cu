@@ -83,8 +83,11 @@ int dalloc(ws_ctx* c, T** p, int64_t count) {
   *p = nullptr;
   if (count <= 0) return WS_OK;
   cudaError_t e = cudaMalloc((void**)p, sizeof(T) * (size_t)count);
-  if (e != cudaSuccess) return fail(c, WS_ECUDA, "cudaMalloc(%lld bytes): %s", (long long)(sizeof(T) * count),
-                                    cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    *p = nullptr;
+    cudaGetLastError();  // reported here, not by the next launch
+    return fail(c, WS_ECUDA, "cudaMalloc(%lld bytes): %s", (long long)(sizeof(T) * count), cudaGetErrorString(e));
+  }
   return WS_OK;
 }
 
@@ -222,15 +225,24 @@ int build_chunks(ws_ctx* c, int config) {
     for (int64_t s0 = 0; s0 < len; s0 += CH)
       items.push_back(TubeItem{off, (int)t, (int)len, (int)s0, (int)items.size(), 0, 0});
   }
-  cudaFree(c->chunks);
-  c->chunks = nullptr;
   const int64_t n = (int64_t)items.size(), nt = c->td.ntubes;
+  // the new blocks first: without them the context keeps those it has
+  TubeItem* chunks = nullptr;
+  unsigned long long* z = nullptr;
   int rc;
-  if ((rc = dalloc(c, &c->chunks, 3 * n))) return rc;
+  if ((rc = dalloc(c, &chunks, 3 * n))) return rc;
+  if ((rc = dalloc(c, &z, 1 + nt + 4 + n))) {
+    cudaFree(chunks);
+    return rc;
+  }
+  if (c->graph_exec) {  // holds the addresses that go
+    cudaGraphExecDestroy(c->graph_exec);
+    c->graph_exec = nullptr;
+  }
+  cudaFree(c->chunks);
+  c->chunks = chunks;
   // nbad, lmax and the counters lie in one block; the first call brings the
   // first two over from their own
-  unsigned long long* z = nullptr;
-  if ((rc = dalloc(c, &z, 1 + nt + 4 + n))) return rc;
   if (c->zeroed) {
     cudaFree(c->zeroed);
   } else {
@@ -1361,10 +1373,6 @@ int ws_autotune(ws_ctx* c, const double* U, int steps, int* choice) {
   cudaFree(Ut);
   if (rc) return rc;
   if ((rc = build_chunks(c, bestc))) return rc;
-  if (c->graph_exec) {
-    cudaGraphExecDestroy(c->graph_exec);
-    c->graph_exec = nullptr;
-  }
   if (choice) *choice = bestc;
   return WS_OK;
 }

@@ -233,8 +233,9 @@ __device__ __forceinline__ void fix_add(float a, float b, int& hi, int& lo) {
 // column, and each adds up its parameters' contributions over the tile's
 // samples in registers, which reach global memory once per CTA.  (One thread per
 // sample adding 1889 shared-memory atomics to the same addresses as its
-// neighbours took 2.71 ms for 65536 samples; this takes 0.1 ms, bound by
-// the float-to-integer conversions, one per sample and parameter.)
+// neighbours took 2.71 ms for 65536 samples; this takes 0.09 ms.  Its warps are
+// few: 150 registers and 93 KB of shared memory a CTA leave 11 % of them on an SM,
+// which issues in 46 % of its cycles.)
 constexpr int GT = 128, GR = NH / (GT / 32), GP = NH + 1;  // GP: row pitch without bank conflicts
 struct GradSmem {
   float W[(NPARAM + 3) / 4 * 4];
